@@ -118,15 +118,18 @@ typedef struct {
                                handle); 0: the built-in defaults */
   int fft_variant;          /* 0 (default): as autotune says.  Otherwise a forced variant,
                                100000 f + 10000 e + 1000 a + 100 b + 10 c + d: a = inverse column
-                               stage (1 persistent, TMA-fed; 2 ping-pong; 3 in-place), b = row
-                               stage (1 ping-pong; 2 in-place), c, d = column and row tiles 1, 2
-                               or 4 times narrower than the widest, f, e = radix plans of the
-                               ping-pong column and row passes (0: larger radices first,
+                               stage (1 persistent, TMA-fed; 2 register-resident two-pass
+                               transforms, the forward stage with it; 3 in-place), b = row
+                               stage (1 register-resident; 2 in-place), c, d = column and row
+                               tiles 1, 2 or 4 times narrower than the widest, f = radix plan of
+                               the TMA-fed stage's passes (0: larger radices first,
                                1024 = 16 x 8 x 8; 1: ascending, 8 x 8 x 16; 2: radix 32 first
-                               for lengths 512 and 1024, 32 x 32).  wf_problem_variant reports
+                               for lengths 512 and 1024, 32 x 32), e carried only: the row stage
+                               has no radix plans.  wf_problem_variant reports
                                the one in use: a = 1 becomes 2 on maps whose column tile is
                                wider than 128 values (few rows, many columns), which one TMA box
-                               cannot hold. */
+                               cannot hold.  The objective's own passes (wf_eval, refreshes,
+                               data synthesis) always run the register-resident stages. */
   int history;              /* 0 (default): off.  k > 0: every map keeps a device ring of its
                                last k iterations' records (k, chi2, |g|/|g0|, step, evals), the
                                convergence trace the paper plots (Sec. 3, Fig. of chi2 against
@@ -354,13 +357,14 @@ wf_status wf_solver_history(const wf_problem* p, double* out, int* counts);
  * shape of a heterogeneous batch (Sec. 2.2; the simulations of Sec. 2.5 need
  * not share a size).  Every problem is started on its own internal stream,
  * ordered after opts->stream (first gradient).  When 2 to 8 problems share
- * the precision and C and opts->fft_variant is 0, each L-BFGS iteration of
- * the whole batch is one set of seven shared launches: every launch covers
- * the blocks of every problem's own grid, each block running the
- * single-problem kernel at its place in its problem's grid, every problem on
- * the ping-pong column and row stages with radix plan 0 and its own tile
- * widths (tuned per shape when opts->autotune, else the widest: variant
- * 2111), so each map ends exactly where its problem solved alone with the
+ * the precision and C and opts->fft_variant is 0, the streaming kernels and
+ * the scalar step of each L-BFGS iteration are launches shared by the whole
+ * batch: every launch covers the blocks of every problem's own grid, each
+ * block running the single-problem kernel at its place in its problem's grid;
+ * the FFT stages are launched per problem, every problem on the
+ * register-resident stages with its own tile widths (tuned per shape when
+ * opts->autotune, else the widest: variant 2111), so each map ends exactly
+ * where its problem solved alone with the
  * variant its stats report ends.  Otherwise every problem is tuned and
  * runs its own kernels, a parallel branch per problem.  opts->check_every
  * iterations are captured in one CUDA graph, so that each round of the batch

@@ -60,15 +60,32 @@ static void wf_geo_tiles(WfGeo& g, int tc_div, int rb_div) {
   if (rb < 1) rb = 1;
   g.RB = rb;
   g.nrb = g.C * g.n / rb;
+  if (g.colinv_kind == WF_COLINV_REG_K) {
+    int tc = wf_rg_tc(g.n, g.C, tc_div);
+    while ((g.h + tc - 1) / tc > g.maxblk) tc *= 2;
+    g.TC = tc;
+    g.ntile = (g.h + tc - 1) / tc;  // one tile, partly empty, where it is wider than the map
+  }
+  if (g.row_kind == WF_ROW_REG_K) {  // eight warps a block, or 1/2 and 1/4 of them
+    const int per = wf_rg_rows(g.nx), need = (g.C * g.n + per - 1) / per;
+    int warps = 8 / rb_div;
+    while (warps > need) warps /= 2;
+    while (warps < 8 && (need + warps - 1) / warps > g.maxblk) warps *= 2;
+    g.RB = per * warps;
+    g.nrb = (need + warps - 1) / warps;
+  }
   g.tc_div = tc_div;
   g.rb_div = rb_div;
 }
 
 // A TMA box spans at most 256 elements per dimension: a column tile wider
 // than 128 complex values (a map of few rows and many columns) cannot be one
-// box row, so such shapes run the inverse column stage on ping-pong passes.
+// box row, so such shapes run the inverse column stage in registers.
 static void wf_geo_fix_kind(WfGeo& g) {
-  if (g.colinv_kind == WF_COLINV_TMA_K && 2 * g.TC > 256) g.colinv_kind = WF_COLINV_PP_K;
+  if (g.colinv_kind == WF_COLINV_TMA_K && 2 * g.TC > 256) {
+    g.colinv_kind = WF_COLINV_REG_K;
+    wf_geo_tiles(g, g.tc_div, g.rb_div);
+  }
 }
 
 WfGeo wf_make_geo(int ny, int nx, int C, int B) {
@@ -92,25 +109,39 @@ WfGeo wf_make_geo(int ny, int nx, int C, int B) {
   if (B > 0)
     while (g.sgroup > 1 && (long long)B * ((nchunk + g.sgroup - 1) / g.sgroup) < WF_STREAM_MIN_BLOCKS) g.sgroup /= 2;
   g.ncomb = (nchunk + g.sgroup - 1) / g.sgroup;
-  wf_geo_tiles(g, WF_TUNE_MAXDIV, WF_TUNE_MAXDIV);  // the narrowest tiles set the stride
+  // the stride of the partial sums covers the narrowest in-place tiles and the
+  // widest register-resident ones (wf_geo_tiles keeps narrower ones within it)
+  g.colinv_kind = WF_COLINV_INPLACE_K;
+  g.row_kind = WF_ROW_INPLACE_K;
+  g.col_plan = g.row_plan = 0;
+  wf_geo_tiles(g, WF_TUNE_MAXDIV, WF_TUNE_MAXDIV);
   g.maxblk = g.ntile > g.nrb ? g.ntile : g.nrb;
   if (g.ncomb > g.maxblk) g.maxblk = g.ncomb;
+  const int wide = wf_rg_tc(ny, C, 1), tiles = (g.h + wide - 1) / wide;
+  if (tiles > g.maxblk) g.maxblk = tiles;
+  g.colinv_kind = WF_COLINV_REG_K;
+  g.row_kind = WF_ROW_REG_K;
   wf_geo_tiles(g, 1, 1);
-  g.colinv_kind = WF_COLINV_TMA ? WF_COLINV_TMA_K : WF_COLINV_PP_K;
-  g.row_kind = WF_ROW_PP_K;
-  g.col_plan = g.row_plan = 0;
-  wf_geo_fix_kind(g);
+  return g;
+}
+
+WfGeo wf_make_geo_pass(int ny, int nx, int C, int B) {
+  WfGeo g = wf_make_geo(ny, nx, C, B);
+  const int fill = 2 * WF_SMS;  // two blocks per SM
+  int tc_div = 1, rb_div = 1;
+  while (tc_div < WF_TUNE_MAXDIV && (long long)B * g.ntile < fill) wf_geo_tiles(g, tc_div *= 2, rb_div);
+  while (rb_div < WF_TUNE_MAXDIV && (long long)B * g.nrb < fill) wf_geo_tiles(g, tc_div, rb_div *= 2);
   return g;
 }
 
 WfGeo wf_geo_variant(const WfGeo& base, int colinv_kind, int row_kind, int tc_div, int rb_div, int col_plan,
                      int row_plan) {
   WfGeo g = base;
-  wf_geo_tiles(g, tc_div, rb_div);
   g.colinv_kind = colinv_kind;
   g.row_kind = row_kind;
   g.col_plan = col_plan;
   g.row_plan = row_plan;
+  wf_geo_tiles(g, tc_div, rb_div);
   wf_geo_fix_kind(g);
   return g;
 }
@@ -304,6 +335,7 @@ extern "C" wf_status wf_problem_create_rect(wf_handle* h, const wf_map* maps, in
   p->precision = precision;
   p->m = lbfgs_m;
   p->g = wf_make_geo(ny, nx, C, count);
+  p->gp = wf_make_geo_pass(ny, nx, C, count);
   p->elt = precision == WF_FP64 ? sizeof(double) : sizeof(float);
   int shared = 1;
   for (int i = 1; i < count; ++i) shared &= maps[i].P == maps[0].P;
@@ -378,7 +410,6 @@ WfBufs wf_bufs(const wf_problem* p) {
   b.scratch = p->scratch;
   b.part = p->part;
   b.tw = p->precision == WF_FP64 ? p->h->tw64 : p->h->tw32;
-  b.ticket = p->flags + 2;  // flags[0] holds the input checks
   b.B = p->count;
   return b;
 }
@@ -396,7 +427,7 @@ extern "C" wf_status wf_eval(wf_problem* p, const void* s, void* grad, double* c
   if (!p || !s || !grad) return wf_fail(WF_EINVAL, "wf_eval: null argument");
   if (s == grad) return wf_fail(WF_EINVAL, "wf_eval: s and grad must not alias");
   WfBufs b = wf_bufs(p);
-  cudaError_t e = WF_DISPATCH(p, wf_launch_eval)(p->g, b, WF_ROW_DATA, WF_IN_STD, s, grad, chi2,
+  cudaError_t e = WF_DISPATCH(p, wf_launch_eval)(p->gp, b, WF_ROW_DATA, WF_IN_STD, s, grad, chi2,
                                                  (cudaStream_t)stream);
   return e == cudaSuccess ? WF_OK : wf_cuda_fail(e, "wf_eval");
 }
@@ -405,7 +436,7 @@ extern "C" wf_status wf_hess_vec(wf_problem* p, const void* v, void* hv, void* s
   if (!p || !v || !hv) return wf_fail(WF_EINVAL, "wf_hess_vec: null argument");
   if (v == hv) return wf_fail(WF_EINVAL, "wf_hess_vec: v and hv must not alias");
   WfBufs b = wf_bufs(p);
-  cudaError_t e = WF_DISPATCH(p, wf_launch_eval)(p->g, b, WF_ROW_NODATA, WF_IN_STD, v, hv, nullptr,
+  cudaError_t e = WF_DISPATCH(p, wf_launch_eval)(p->gp, b, WF_ROW_NODATA, WF_IN_STD, v, hv, nullptr,
                                                  (cudaStream_t)stream);
   return e == cudaSuccess ? WF_OK : wf_cuda_fail(e, "wf_hess_vec");
 }
@@ -413,7 +444,7 @@ extern "C" wf_status wf_hess_vec(wf_problem* p, const void* v, void* hv, void* s
 extern "C" wf_status wf_signal_map(wf_problem* p, const void* s, void* x, void* stream) {
   if (!p || !s || !x) return wf_fail(WF_EINVAL, "wf_signal_map: null argument");
   WfBufs b = wf_bufs(p);
-  cudaError_t e = WF_DISPATCH(p, wf_launch_signal)(p->g, b, WF_IN_STD, s, x, (cudaStream_t)stream);
+  cudaError_t e = WF_DISPATCH(p, wf_launch_signal)(p->gp, b, WF_IN_STD, s, x, (cudaStream_t)stream);
   return e == cudaSuccess ? WF_OK : wf_cuda_fail(e, "wf_signal_map");
 }
 
@@ -421,7 +452,7 @@ extern "C" wf_status wf_simulate_data(wf_problem* p, const void* z, const void* 
                                       void* stream) {
   if (!p || !z || !noise || !d_out) return wf_fail(WF_EINVAL, "wf_simulate_data: null argument");
   WfBufs b = wf_bufs(p);
-  cudaError_t e = WF_DISPATCH(p, wf_launch_simulate)(p->g, b, z, noise, d_out, (cudaStream_t)stream);
+  cudaError_t e = WF_DISPATCH(p, wf_launch_simulate)(p->gp, b, z, noise, d_out, (cudaStream_t)stream);
   return e == cudaSuccess ? WF_OK : wf_cuda_fail(e, "wf_simulate_data");
 }
 
@@ -477,7 +508,7 @@ extern "C" wf_status wf_eval_bands(wf_problem* p, const void* s, void* grad, dou
   wf_status rs = band_partials(p, n_b);
   if (rs != WF_OK) return rs;
   WfBufs b = wf_bufs(p);
-  cudaError_t e = WF_DISPATCH(p, wf_launch_eval_bands)(p->g, b, s, grad, chi2, band, n_b, p->bpart, dlogq,
+  cudaError_t e = WF_DISPATCH(p, wf_launch_eval_bands)(p->gp, b, s, grad, chi2, band, n_b, p->bpart, dlogq,
                                                        (cudaStream_t)stream);
   return e == cudaSuccess ? WF_OK : wf_cuda_fail(e, "wf_eval_bands");
 }

@@ -20,7 +20,8 @@ struct WfSolver;  // L-BFGS state, allocated on the first solve (wf_solve.cu)
 struct wf_problem {
   wf_handle* h;
   int count, n, nx, C, dtype, precision, m;  // n = ny rows of nx pixels
-  WfGeo g;
+  WfGeo g;               // of the solver's launches (the variant its last start chose)
+  WfGeo gp;              // of the objective's passes
   size_t elt;            // bytes of the working type
   int sp_shared;         // one sqrt(P) table serves every map
   long long sp_stride;   // elements between maps' sqrt(P) tables

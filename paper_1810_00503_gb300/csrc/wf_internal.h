@@ -51,7 +51,9 @@ __device__ __forceinline__ long long wf_chk(long long i, long long lim, int line
     return cudaSuccess;                                                        \
   }
 #endif
-#define WF_DBG_TUS(X) X(ops_f32) X(ops_f64) X(lbcol_f32) X(lbcol_f64) X(lbrow_f32) X(lbrow_f64) X(solve) X(noalloc) X(bandpower) X(multi) X(any)
+#define WF_DBG_TUS(X) X(ops_f32) X(ops_f64) X(lbcol_f32) X(lbcol_f64) X(lbrow_f32) X(lbrow_f64) X(solve) X(noalloc) X(bandpower) X(multi) X(any) \
+  X(reg_f32_small) X(reg_f32_256) X(reg_f32_512) X(reg_f32_1024) X(reg_f64_small) X(reg_f64_256) X(reg_f64_512) \
+  X(reg_f64_1024)
 #define WF_DBG_DECL(name) cudaError_t wf_dbg_read_##name(unsigned long long* out, int reset);
 WF_DBG_TUS(WF_DBG_DECL)
 
@@ -65,7 +67,8 @@ WF_DBG_TUS(WF_DBG_DECL)
 #define WF_NPLAN 3
 #define WF_TWTAB_ALL (WF_NPLAN * WF_TWTAB)
 
-// Radix plans of the ping-pong FFT passes (the in-place passes use plan 0):
+// Radix plans of the passes of the TMA-fed inverse column stage (the in-place
+// passes use plan 0, the register-resident stages have none):
 //   0: ceil(lgL / 4) passes, the bits spread evenly, larger radices first
 //      (1024 = 16 x 8 x 8, 512 = 8 x 8 x 8, 256 = 16 x 16, 128 = 16 x 8);
 //   1: the same radices in ascending order (1024 = 8 x 8 x 16, 128 = 8 x 16);
@@ -75,9 +78,6 @@ WF_DBG_TUS(WF_DBG_DECL)
 __host__ __device__ inline int wf_plan_np(int lgL, int plan) {
   return (plan == 2 && lgL >= 9) ? 2 : (lgL + 3) >> 2;
 }
-// Kernels are instantiated per plan; those with radix-32 passes (plan 2) are
-// compiled for two blocks per SM (FP32) to hold the 32 values.
-#define WF_MINB_PLAN(T, PLAN) ((PLAN) == 2 ? (sizeof(T) == 4 ? 2 : 1) : WF_MINB(T))
 __host__ __device__ inline int wf_plan_bits(int lgL, int plan, int p) {
   if (plan == 2 && lgL >= 9) return p == 0 ? 5 : lgL - 5;
   const int np = (lgL + 3) >> 2;
@@ -109,36 +109,8 @@ __host__ __device__ inline int wf_plan_bits(int lgL, int plan, int p) {
 #define WF_STREAM_GROUP 8
 #endif
 #define WF_STREAM_MIN_BLOCKS 2048
-// FFT stages of the L-BFGS iteration on ping-pong passes with direct global
-// input/output (1) or on in-place shared-memory passes (0).
-#ifndef WF_FFT_PP
-#define WF_FFT_PP 1
-#endif
-// Inverse column stage of the iteration as a persistent kernel fed by TMA (1)
-// or one block per tile (0, also used when the driver lacks the tensor-map
-// encoder).  The row and forward column stages stay one block per tile: their
-// persistent TMA-fed forms measured slower (0.66 vs 0.59 ms, 0.93 vs 0.80 ms
-// on the 120 x 1024^2 batch).
-#ifndef WF_COLINV_TMA
-#define WF_COLINV_TMA 1
-#endif
-
-// Work queue for the objective pass's inverse column stage: the resident
-// blocks take (map, tile) items from an atomic counter, in order, each claiming
-// its next item before it transforms the current one and asking L2 for that
-// item's rows (1.63 ms per 120 x 1024^2 pass against 1.69 with the items taken
-// round-robin).
-#ifndef WF_COLINV_QUEUE
-#define WF_COLINV_QUEUE 1
-#endif
-
-// Items ahead whose rows the objective pass's persistent inverse column stage
-// asks L2 for (one: 1.70 ms per 120 x 1024^2 pass; two: 1.75; three: 1.77).
-#ifndef WF_COLINV_AHEAD
-#define WF_COLINV_AHEAD 1
-#endif
-
-// Resident blocks per SM requested from the compiler for the FFT-stage kernels.
+#define WF_SMS 152  // streaming multiprocessors of the chip
+// Resident blocks per SM requested from the compiler for the in-place FFT stages.
 // FP32: three blocks of 256 threads (85 registers a thread; the radix-16 passes
 // spill a few hundred bytes to L1-resident local memory, and the extra resident
 // warps still win over two blocks by 8-17% per stage).  FP64: one block.
@@ -146,17 +118,7 @@ __host__ __device__ inline int wf_plan_bits(int lgL, int plan, int p) {
 #define WF_MINB32 3
 #endif
 #define WF_MINB(T) (sizeof(T) == 4 ? WF_MINB32 : 1)
-// The same for the objective pass's forward column stage (k_col_fwd): its tile
-// and tables take 40 KB of shared memory, so four blocks fit, and at 64
-// registers it does not spill (1.67 against 1.73 ms for the 120 x 1024^2 pass;
-// five blocks, 48 registers: 1.76 ms).  Two channels keep three blocks (at 64
-// registers they spill).  The iteration's forward stage has its own setting
-// below.
-#ifndef WF_MINB_COLFWD32
-#define WF_MINB_COLFWD32 4
-#endif
-#define WF_MINB_COLFWD(T, C) (sizeof(T) == 4 ? ((C) == 1 ? WF_MINB_COLFWD32 : WF_MINB32) : 1)
-// The iteration's forward column stage (k_lb_colfwd): blocks per SM, and the
+// The iteration's in-place forward column stage (k_lb_colfwd): blocks per SM, and the
 // groups its epilogue takes its rows of p and g in.  Four groups fit 64
 // registers without spills at four blocks per SM: 0.668 against 0.683 ms (one
 // group, 80 registers, three blocks) on 120 x 1024^2.  Two channels (E/B) keep
@@ -256,8 +218,8 @@ __device__ __forceinline__ void wf_warp_bin_add(double* bins, int l, double v) {
 // length-nx real transforms.
 // Kernel variants of the L-BFGS FFT stages, chosen per shape by the autotuner
 // (wf_solve.cu) or forced through wf_opts.fft_variant.
-enum { WF_COLINV_TMA_K = 1, WF_COLINV_PP_K = 2, WF_COLINV_INPLACE_K = 3 };
-enum { WF_ROW_PP_K = 1, WF_ROW_INPLACE_K = 2 };
+enum { WF_COLINV_TMA_K = 1, WF_COLINV_REG_K = 2, WF_COLINV_INPLACE_K = 3 };
+enum { WF_ROW_REG_K = 1, WF_ROW_INPLACE_K = 2 };
 #define WF_TUNE_MAXDIV 4  // tiles may be 1, 2 or 4 times narrower than the widest
 
 struct WfGeo {
@@ -271,13 +233,28 @@ struct WfGeo {
   int maxblk;      // stride of the partial-sum slots: covers every tile choice
   int colinv_kind, row_kind;  // WF_COLINV_*_K, WF_ROW_*_K
   int tc_div, rb_div;         // TC and RB are the widest tile divided by these (1, 2, 4)
-  int col_plan, row_plan;     // radix plans of the ping-pong column and row passes (0..WF_NPLAN-1)
+  int col_plan, row_plan;     // radix plan of the TMA-fed stage's passes; row_plan is carried only (0..WF_NPLAN-1)
 };
 
-// Widest tiles and the default kernel variants.
-// B: maps per launch, which sets the streaming kernels' chunk groups (0: many).
-WfGeo wf_make_geo(int ny, int nx, int C, int B = 0);
-inline WfGeo wf_make_geo(int n, int C) { return wf_make_geo(n, n, C); }
+// The register-resident stages (wf_reg.cuh) with their widest tiles; B: maps per
+// launch, which sets the streaming kernels' chunk groups (0: many).
+WfGeo wf_make_geo(int ny, int nx, int C, int B);
+// The same with tiles narrowed for a batch too small to fill the chip with the
+// widest: what the objective's passes run (the L-BFGS stages are tuned).
+WfGeo wf_make_geo_pass(int ny, int nx, int C, int B);
+
+// Register-resident stages.  Widest tile: wf_rg_seq(N) sequences a block (256
+// threads from 64 rows up; 64-byte rows of a tile at 1024, 128-byte rows and
+// more below), and 1/2 and 1/4 of it.
+__host__ __device__ constexpr int wf_rg_seq(int N) { return N == 1024 ? 8 : N >= 256 ? 16 : 32; }
+__host__ __device__ constexpr int wf_rg_tc(int N, int C, int div) {
+  const int seq = N == 8 && div == 4 ? 16 : wf_rg_seq(N) / div;  // at least a warp a block
+  return seq / C < 2 ? 2 : seq / C;
+}
+// Rows a warp of the row stage takes: pairs of rows, 32 or fewer values a thread.
+__host__ __device__ constexpr int wf_rg_rows(int nx) {
+  return nx == 1024 ? 2 : nx >= 256 ? 4 : nx >= 64 ? 8 : nx >= 16 ? 16 : 32;
+}
 // Blocks per map of the band reductions: about 4096 modes each, at most 64.
 inline int wf_band_nblk(const WfGeo& g) {
   const long long nsp = (long long)g.C * g.n * (g.h + 1);
@@ -297,8 +274,6 @@ struct WfBufs {
   void* scratch;      // [B][C][ny][h] complex: between the column and row stages
   double* part;       // [B][WF_NSLOT][maxblk]
   const void* tw;     // twiddle table, WF_NT complex of type T
-  int* ticket;        // device counter of the objective pass's inverse column stage
-                      // work queue (nullptr: that stage runs its round-robin form)
   int B;
 };
 
@@ -343,8 +318,9 @@ struct WfLbBufs {
   int inject_map;   // map whose tile copies are never issued (-1: none), see wf_opts
   long long spin_limit;  // bound of device waits, SM cycles
 };
-// Launches shared by several problems (wf_map_solve_many: one problem per map
-// shape of a heterogeneous batch).  Every problem keeps its own geometry,
+// Streaming launches shared by several problems (wf_map_solve_many: one problem
+// per map shape of a heterogeneous batch; the FFT stages, whose code differs by
+// length, are launched per problem).  Every problem keeps its own geometry,
 // buffers and L-BFGS state; a shared launch covers the blocks of every
 // problem's own grid, problem q's at blocks start[q] .. start[q+1] - 1, and
 // each block runs the single-problem kernel body at its coordinates in its
@@ -357,18 +333,12 @@ struct WfMultiArgs {
   WfBufs b[WF_MULTI_MAX];
   WfLbBufs lb[WF_MULTI_MAX];
 };
-// FFT-stage variant the shared launches run (ping-pong inverse column and row
-// stages, radix plan 0; the widest tiles here, the tile widths tuned per
-// problem when the solve autotunes).
+// FFT-stage variant of a shared batch: the register-resident stages (the widest
+// tiles here, the widths tuned per problem when the solve autotunes).
 #define WF_MULTI_VARIANT 2111
+#define WF_TMA_VARIANT 1111  // the TMA-fed inverse column stage, widest tiles
 template <typename T>
 cudaError_t wf_launch_multi_comb(const WfMultiArgs& a, int mode, cudaStream_t st);
-template <typename T>
-cudaError_t wf_launch_multi_colinv(const WfMultiArgs& a, cudaStream_t st);
-template <typename T>
-cudaError_t wf_launch_multi_row(const WfMultiArgs& a, cudaStream_t st);
-template <typename T>
-cudaError_t wf_launch_multi_colfwd(const WfMultiArgs& a, cudaStream_t st);
 template <typename T>
 cudaError_t wf_launch_multi_qdots(const WfMultiArgs& a, cudaStream_t st);
 
@@ -382,6 +352,22 @@ template <typename T>
 cudaError_t wf_launch_lb_colfwd(const WfGeo& g, const WfBufs& b, const WfLbBufs& lb, cudaStream_t st);
 template <typename T>
 cudaError_t wf_launch_lb_qdots(const WfGeo& g, const WfBufs& b, const WfLbBufs& lb, cudaStream_t st);
+// Register-resident two-pass stages (wf_reg.cuh) of one length: N the column
+// length (ny), NX the row length, tiles g.TC and g.RB.
+template <typename T, int N>
+cudaError_t wf_reg_colinv(const WfGeo& g, const WfBufs& b, int in_layout, const void* src, cudaStream_t st);
+template <typename T, int N>
+cudaError_t wf_reg_colfwd(const WfGeo& g, const WfBufs& b, int in_layout, const void* src, void* dst, cudaStream_t st);
+template <typename T, int N>
+cudaError_t wf_reg_colsim(const WfGeo& g, const WfBufs& b, cudaStream_t st);
+template <typename T, int N>
+cudaError_t wf_reg_lb_colinv(const WfGeo& g, const WfBufs& b, const WfLbBufs& lb, cudaStream_t st);
+template <typename T, int N>
+cudaError_t wf_reg_lb_colfwd(const WfGeo& g, const WfBufs& b, const WfLbBufs& lb, cudaStream_t st);
+template <typename T, int NX>
+cudaError_t wf_reg_row(const WfGeo& g, const WfBufs& b, int mode, const void* aux, void* out, cudaStream_t st);
+template <typename T, int NX>
+cudaError_t wf_reg_lb_row(const WfGeo& g, const WfBufs& b, const WfLbBufs& lb, cudaStream_t st);
 // Full objective+gradient pass on packed vectors (src -> dst), all maps.
 template <typename T>
 cudaError_t wf_launch_eval_pk(const WfGeo& g, const WfBufs& b, const void* src, void* dst, cudaStream_t st);

@@ -17,8 +17,8 @@
 // packed half plane (1 on the packed column 0, 2 elsewhere), which equal the
 // full-plane real inner product.
 #pragma once
+#include "wf_fft_pp.cuh"
 #include "wf_ops.cuh"
-#include "wf_stage_pp.cuh"
 #include "wf_tma.cuh"
 
 
@@ -375,27 +375,41 @@ k_lb_qdots(WfGeo g, WfLbBufs lb, double* part) {
 // ---------------------------------------------------------------------------
 // Column stages of the Hessian-vector product on p = P[next] of each map.
 // ---------------------------------------------------------------------------
-// One block per column tile; KIND WF_COLINV_PP_K (ping-pong passes) or
-// WF_COLINV_INPLACE_K (in-place passes).
-template <typename T, int C, int KIND, int PLAN>
-__device__ __forceinline__ void wf_lb_colinv(const WfGeo& g, const T* sp_, long long sp_stride, void* scratch_,
-                                             const void* tw_, const WfLbBufs& lb, const WfBlk kb) {
-  const int b = kb.y;
+// One block per column tile, in-place passes (the register-resident form is
+// k_rg_lb_colinv in wf_reg_impl.cuh).
+template <typename T, int C>
+__global__ void __launch_bounds__(WF_THREADS, WF_MINB(T))
+k_lb_colinv(WfGeo g, const T* sp_, long long sp_stride, void* scratch_, const void* tw_, WfLbBufs lb) {
+  const int b = blockIdx.y;
   const WfLbMap* M = lb.st + b;
   if (!M->active) return;
   const size_t vsz = (size_t)C * g.n * g.h;
-  const V2<T>* p = (const V2<T>*)lb.ring + ((size_t)M->next * kb.ny + b) * vsz;
-  if constexpr (KIND == WF_COLINV_PP_K)
-    wf_col_inv_pp<T, C, WF_IN_PK, PLAN>(g, p, sp_ + (size_t)b * sp_stride, (V2<T>*)scratch_ + (size_t)b * vsz, tw_,
-                                        kb.x * g.TC);
-  else
-    wf_col_inv_body<T, C, WF_IN_PK>(g, p, sp_ + (size_t)b * sp_stride, (V2<T>*)scratch_ + (size_t)b * vsz, tw_,
-                                    kb.x * g.TC);
+  const V2<T>* p = (const V2<T>*)lb.ring + ((size_t)M->next * gridDim.y + b) * vsz;
+  wf_col_inv_body<T, C, WF_IN_PK>(g, p, sp_ + (size_t)b * sp_stride, (V2<T>*)scratch_ + (size_t)b * vsz, tw_,
+                                  blockIdx.x * g.TC);
 }
-template <typename T, int C, int KIND, int PLAN>
-__global__ void __launch_bounds__(WF_THREADS, WF_MINB_PLAN(T, PLAN))
-k_lb_colinv(WfGeo g, const T* sp_, long long sp_stride, void* scratch_, const void* tw_, WfLbBufs lb) {
-  wf_lb_colinv<T, C, KIND, PLAN>(g, sp_, sp_stride, scratch_, tw_, lb, wf_blk());
+
+// Packed value of column tile element (row j, channel c, column kx) after the
+// per-mode operator (R(k) sqrt(P)/n, or its adjoint), read through `ld(cc, row)`
+// (channel cc's packed value at row `row` of this column).  Column 0 is
+// unpacked with row ny - j, the operator applied at kx = 0 and kx = nx/2, and
+// packed again.
+template <typename T, int C, bool ADJ, class LD>
+__device__ __forceinline__ V2<T> wf_mode_packed(LD& ld, int j, int c, int kx, const WfGeo& g, const T* sp) {
+  V2<T> v[C];
+  if (kx != 0) {
+#pragma unroll
+    for (int cc = 0; cc < C; ++cc) v[cc] = ld(cc, j);
+    wf_mode_op<T, C, ADJ>(v, j, kx, g, sp, (T)1);
+    return v[c];
+  }
+  const int jm = (g.n - j) & (g.n - 1);
+  V2<T> X0[C], Xh[C];
+#pragma unroll
+  for (int cc = 0; cc < C; ++cc) wf_unpack0<T>(ld(cc, j), ld(cc, jm), X0[cc], Xh[cc]);
+  wf_mode_op<T, C, ADJ>(X0, j, 0, g, sp, (T)1);
+  wf_mode_op<T, C, ADJ>(Xh, j, g.h, g, sp, (T)1);
+  return wf_pack0<T>(X0[c], Xh[c]);
 }
 
 // Persistent inverse column stage with the next tile prefetched by TMA.
@@ -404,7 +418,7 @@ k_lb_colinv(WfGeo g, const T* sp_, long long sp_stride, void* scratch_, const vo
 // round-robin by the resident blocks; while a block runs the second and third
 // FFT passes of one tile, the copy engine brings in the next tile, whose first
 // pass then reads shared memory (the per-mode operator R sqrt(P)/n applied on
-// the way in, as in wf_col_inv_pp).  tm: 2-D view of the whole history ring,
+// the way in).  tm: 2-D view of the whole history ring,
 // rows of h = nx/2 packed values; the map's direction P[next] is rows
 // ((next B + b) C ny + r).
 template <typename T>
@@ -492,9 +506,11 @@ k_lb_colinv_tma(WfGeo g, const T* sp_, long long sp_stride, void* scratch_, cons
 }
 
 template <typename T, int C>
-__device__ __forceinline__ void wf_lb_colfwd(const WfGeo& g, const T* sp_, long long sp_stride, const void* scratch_,
-                                             const void* tw_, const WfLbBufs& lb, double* part, const WfBlk kb) {
+__global__ void __launch_bounds__(WF_THREADS, WF_MINB_LBCOLFWD(T, C))
+k_lb_colfwd(WfGeo g, const T* sp_, long long sp_stride, const void* scratch_, const void* tw_, WfLbBufs lb,
+            double* part) {
   extern __shared__ __align__(16) unsigned char wf_smem[];
+  const WfBlk kb = wf_blk();
   const int b = kb.y;
   const WfLbMap* M = lb.st + b;
   if (!M->active) return;
@@ -567,21 +583,11 @@ __device__ __forceinline__ void wf_lb_colfwd(const WfGeo& g, const T* sp_, long 
   __syncthreads();
   wf_flush_slots(red, 5, WF_THREADS / 32, ids, part + (size_t)b * WF_NSLOT * g.maxblk, g.maxblk, kb.x);
 }
-template <typename T, int C>
-__global__ void __launch_bounds__(WF_THREADS, WF_MINB_LBCOLFWD(T, C))
-k_lb_colfwd(WfGeo g, const T* sp_, long long sp_stride, const void* scratch_, const void* tw_, WfLbBufs lb,
-            double* part) {
-  wf_lb_colfwd<T, C>(g, sp_, sp_stride, scratch_, tw_, lb, part, wf_blk());
-}
-
-// Row stage of the Hessian-vector product for the maps still iterating.
-// KIND WF_ROW_PP_K (ping-pong passes) or WF_ROW_INPLACE_K (in-place passes).
-template <typename T, int KIND, int PLAN>
-__global__ void __launch_bounds__(WF_THREADS, WF_MINB_PLAN(T, PLAN))
+// Row stage of the Hessian-vector product for the maps still iterating, in-place
+// passes.
+template <typename T>
+__global__ void __launch_bounds__(WF_THREADS, WF_MINB(T))
 k_lb_row(WfGeo g, void* scratch_, const void* w_, double* part, const void* tw_, const WfLbMap* st) {
   if (!st[blockIdx.y].active) return;
-  if constexpr (KIND == WF_ROW_PP_K)
-    wf_row_pp<T, WF_ROW_NODATA, PLAN>(g, (V2<T>*)scratch_, nullptr, (const T*)w_, part, tw_);
-  else
-    k_row_body<T, WF_ROW_NODATA>(g, scratch_, nullptr, w_, nullptr, nullptr, part, tw_);
+  k_row_body<T>(g, scratch_, w_, part, tw_);
 }

@@ -77,7 +77,7 @@ __global__ void k_noalloc_sqrtp(const T* P, size_t total, int n, T* sp) {
 template <typename T>
 static wf_status noalloc_impl(unsigned char* base, const void* s, const void* d, const void* w, const void* P,
                               int n, int C, int count, double* chi2, void* grad, cudaStream_t st) {
-  const WfGeo g = wf_make_geo(n, C);
+  const WfGeo g = wf_make_geo_pass(n, n, C, count);
   const size_t elt = sizeof(T);
   const size_t nsp = (size_t)C * n * (n / 2 + 1);
   const size_t off_sp = WF_NOALLOC_DATA;
@@ -103,7 +103,6 @@ static wf_status noalloc_impl(unsigned char* base, const void* s, const void* d,
   b.scratch = base + off_scr;
   b.part = (double*)(base + off_part);
   b.tw = base + (sizeof(T) == 8 ? WF_NOALLOC_TW64 : WF_NOALLOC_TW32);
-  b.ticket = nullptr;
   b.B = count;
   e = wf_launch_eval<T>(g, b, WF_ROW_DATA, WF_IN_STD, s, grad, chi2, st);
   return e == cudaSuccess ? WF_OK : wf_cuda_fail(e, "wf_eval_noalloc");

@@ -4,14 +4,14 @@
 // nx pixels, h = nx/2 packed columns) is three stages:
 //   inverse column stage: load a tile of packed spectrum columns, multiply by
 //     R(k) sqrt(P)/n (step A1), inverse FFT along y (first half of A2), store
-//     the tile to scratch (k_col_inv; the ping-pong form k_col_inv_pp_pers in
-//     wf_stage_pp.cuh);
+//     the tile to scratch;
 //   row stage: c2r along x (rest of A2), pixel residual r = d - x, wr = w r
 //     and the data term sum r w r (A3), r2c of wr along x (first half of A4),
-//     store back to scratch (k_row; k_row_pp in wf_stage_pp.cuh);
+//     store back to scratch;
 //   forward column stage: forward FFT along y (rest of A4), sqrt(P) R(k)^T / n
-//     (adjoint, A5), g = 2 (s - .), prior term sum |s|^2, store g
-//     (k_col_fwd).
+//     (adjoint, A5), g = 2 (s - .), prior term sum |s|^2, store g.
+// wf_reg.cuh has their kernels; the in-place forms here and the TMA-fed inverse
+// column stage (wf_lbfgs.cuh) are further variants for the L-BFGS iteration.
 // Spectra are held in a packed half-plane layout [ny][nx/2] in which column 0
 // carries the two self-conjugate columns kx = 0 and kx = nx/2 as X0 + i Xh;
 // the column FFT of that packed column is then an ordinary complex FFT whose
@@ -367,15 +367,6 @@ __device__ __forceinline__ void wf_col_inv_body(const WfGeo& g, const V2<T>* src
   wf_tile_store_pk<T, C>(scr, buf, n, g.h, lgTC, kx0);
 }
 
-template <typename T, int C, int IN>
-__global__ void __launch_bounds__(WF_THREADS, WF_MINB(T))
-k_col_inv(WfGeo g, const void* src_, const T* sp_, long long sp_stride, void* scratch_, const void* tw_) {
-  const int b = blockIdx.y, n = g.n, h = g.h;
-  const size_t sstride = (size_t)C * n * (IN == WF_IN_PK ? h : h + 1);
-  wf_col_inv_body<T, C, IN>(g, (const V2<T>*)src_ + (size_t)b * sstride, sp_ + (size_t)b * sp_stride,
-                            (V2<T>*)scratch_ + (size_t)b * C * n * h, tw_);
-}
-
 // Forward column stage shared by the gradient and Hessian-vector epilogues:
 // scratch tile at packed column kx0 -> forward FFT along y -> sqrt(P) R^T / n,
 // left in buf.
@@ -389,89 +380,6 @@ __device__ __forceinline__ void wf_col_fwd_front(const WfGeo& g, const V2<T>* sc
   fft_smem<T, -1, WF_EMAX>(buf, g.lgn, CT, 1, CT, s_tw);
   wf_col_scale<T, C, true>(buf, g, lgTC, kx0, sp, (T)1);
   __syncthreads();
-}
-
-// Epilogue of the forward column stage on a transformed, scaled tile `buf`
-// ([n][C TC], swizzled as the passes that produced it: SWP for the ping-pong
-// passes): out = 2 (src - a) for the tile's columns of src, dst (packed or
-// standard layout); the prior partial sum |src|^2 and |out|^2 with the
-// half-plane weights go to slot `slot_ix` of the map's partial sums part_b.
-template <typename T, int C, int IN, bool SWP>
-__device__ __forceinline__ void wf_col_fwd_out(const WfGeo& g, V2<T>* buf, const V2<T>* src, V2<T>* dst, int kx0,
-                                               double* part_b, int slot_ix) {
-  const int n = g.n, h = g.h, lgn = g.lgn, TC = g.TC, lgTC = __ffs(TC) - 1, CT = C * TC;
-  WfAcc<T> acc = 0, acc2 = 0;  // per-thread partials; FP64 from the block sum on
-  for (int e = threadIdx.x; e < C * n * TC; e += blockDim.x) {
-    const int t = e & (TC - 1), r = e >> lgTC, j = r & (n - 1), c = r >> lgn;
-    const int kx = kx0 + t;
-    const V2<T> sv = wf_load_spec<T, C, IN>(src, c, j, kx, n, h);
-    const V2<T> a = buf[wf_swz<T, SWP>(j * CT + c * TC + t)];
-    const V2<T> o = mk<T>((T)2 * (sv.x - a.x), (T)2 * (sv.y - a.y));
-    const T m2 = sv.x * sv.x + sv.y * sv.y;
-    const T o2 = o.x * o.x + o.y * o.y;
-    acc += (kx == 0) ? m2 : (T)2 * m2;
-    acc2 += (kx == 0) ? o2 : (T)2 * o2;
-    if constexpr (IN == WF_IN_PK) {
-      dst[WF_CHK(((size_t)c * n + j) * h + kx, (size_t)C * n * h)] = o;
-    } else {
-      if (kx == 0) buf[wf_swz<T, SWP>(j * CT + c * TC + t)] = o;
-      else dst[WF_CHK(((size_t)c * n + j) * (h + 1) + kx, (size_t)C * n * (h + 1))] = o;
-    }
-  }
-  if constexpr (IN == WF_IN_STD) {
-    if (kx0 == 0) {
-      __syncthreads();
-      for (int j = threadIdx.x; j < n; j += blockDim.x) {
-        const int jm = (n - j) & (n - 1);
-#pragma unroll
-        for (int c = 0; c < C; ++c) {
-          V2<T> X0, Xh;
-          wf_unpack0<T>(buf[wf_swz<T, SWP>(j * CT + c * TC)], buf[wf_swz<T, SWP>(jm * CT + c * TC)], X0, Xh);
-          V2<T>* row = dst + WF_CHK(((size_t)c * n + j) * (h + 1), (size_t)C * n * (h + 1) - h);
-          row[0] = X0;
-          row[h] = Xh;
-        }
-      }
-    }
-  }
-  const double tot = wf_block_sum((double)acc);
-  if (threadIdx.x == 0) part_b[(size_t)WF_SLOT_PRIOR * g.maxblk + slot_ix] = tot;
-  const double tot2 = wf_block_sum((double)acc2);
-  if (threadIdx.x == 0) part_b[(size_t)WF_SLOT_OUT2 * g.maxblk + slot_ix] = tot2;
-}
-
-// ---------------------------------------------------------------------------
-// k_col_fwd: scratch tile -> forward FFT along y -> sqrt(P) R^T / n = a ->
-// out = 2 (src - a) (the gradient, or the Hessian-vector product when the row
-// stage ran without data); prior partial sum |src|^2 with half-plane weights.
-// One block per column tile.  (Persistent forms, the next tile's rows
-// prefetched, measured slower on 120 x 1024^2: items taken round-robin 1.01 ms
-// against 0.69 ms; items taken in order from an atomic counter, 2.00 ms for
-// the whole objective pass against 1.69 ms.)
-// ---------------------------------------------------------------------------
-template <typename T, int C, int IN>
-__global__ void __launch_bounds__(WF_THREADS, WF_MINB_COLFWD(T, C))
-k_col_fwd(WfGeo g, const void* src_, const T* sp_, long long sp_stride, const void* scratch_,
-          void* dst_, double* part, const void* tw_) {
-  extern __shared__ __align__(16) unsigned char wf_smem[];
-  V2<T>* s_tw = (V2<T>*)wf_smem;
-  V2<T>* buf = s_tw + WF_NT;
-  const int b = blockIdx.y, n = g.n, h = g.h, lgn = g.lgn;
-  const int TC = g.TC, lgTC = __ffs(TC) - 1, CT = C * TC, kx0 = blockIdx.x * TC;
-  const int pitch = IN == WF_IN_PK ? h : h + 1;
-  const size_t sstride = (size_t)C * n * pitch;
-  // the epilogue reads this tile's rows of src after the transform: start them towards L2
-  wf_prefetch_rows((const V2<T>*)src_ + (size_t)b * sstride + kx0, C * n, (size_t)pitch * sizeof(V2<T>),
-                   TC * (int)sizeof(V2<T>));
-  wf_stage_tw<T>(s_tw, (const V2<T>*)tw_, lgn);
-  wf_tile_load<T, C, WF_IN_PK>(buf, (const V2<T>*)scratch_ + (size_t)b * C * n * h, n, h, lgTC, kx0);
-  __syncthreads();
-  fft_smem<T, -1, WF_EMAX>(buf, lgn, CT, 1, CT, s_tw);
-  wf_col_scale<T, C, true>(buf, g, lgTC, kx0, sp_ + (size_t)b * sp_stride, (T)1);
-  __syncthreads();
-  wf_col_fwd_out<T, C, IN, false>(g, buf, (const V2<T>*)src_ + (size_t)b * sstride,
-                                  (V2<T>*)dst_ + (size_t)b * sstride, kx0, part + (size_t)b * WF_NSLOT * g.maxblk,
-                                  blockIdx.x);
 }
 
 // Scale the sqrt(P)/n table by sqrt(q_l) on the modes of band l (others 1):
@@ -489,41 +397,12 @@ __global__ void k_band_scale(const T* sp0, T* sp, size_t nsp, int ntab, const in
 }
 
 // ---------------------------------------------------------------------------
-// k_col_sim: scratch tile holding the row r2c of a white field z -> forward
-// FFT along y -> scale by 1/sqrt(ny nx) (unitary U z) -> R sqrt(P)/n -> inverse FFT
-// along y -> scratch.  Used to synthesise A z for simulations.
+// k_row_body: row stage of the Hessian-vector product on in-place passes, over
+// RB of the C*ny rows of each map (rows of nx pixels): c2r, r = -x, wr = w r,
+// data partial sum r.wr, r2c of wr, store packed rows back to scratch.
 // ---------------------------------------------------------------------------
-template <typename T, int C>
-__global__ void __launch_bounds__(WF_THREADS, WF_MINB(T))
-k_col_sim(WfGeo g, const T* sp_, long long sp_stride, void* scratch_, const void* tw_) {
-  extern __shared__ __align__(16) unsigned char wf_smem[];
-  V2<T>* s_tw = (V2<T>*)wf_smem;
-  V2<T>* buf = s_tw + WF_NT;
-  const int b = blockIdx.y, n = g.n, h = g.h, lgn = g.lgn;
-  const int TC = g.TC, lgTC = __ffs(TC) - 1, CT = C * TC, kx0 = blockIdx.x * TC;
-  wf_stage_tw<T>(s_tw, (const V2<T>*)tw_, lgn);
-  V2<T>* sc = (V2<T>*)scratch_ + (size_t)b * C * n * h;
-  wf_tile_load<T, C, WF_IN_PK>(buf, sc, n, h, lgTC, kx0);
-  __syncthreads();
-  fft_smem<T, -1, WF_EMAX>(buf, lgn, CT, 1, CT, s_tw);
-  const T unit = (T)(1.0 / sqrt((double)n * (double)g.nx));
-  wf_col_scale<T, C, false>(buf, g, lgTC, kx0, sp_ + (size_t)b * sp_stride, unit);
-  __syncthreads();
-  fft_smem<T, +1, WF_EMAX>(buf, lgn, CT, 1, CT, s_tw);
-  wf_tile_store_pk<T, C>(sc, buf, n, h, lgTC, kx0);
-}
-
-// ---------------------------------------------------------------------------
-// k_row: row stage over RB of the C*ny rows of each map (rows of nx pixels).
-//   MODE DATA / NODATA: c2r, r = d - x (or -x), wr = w r, data partial sum
-//     r.wr, r2c of wr, store packed rows back to scratch.
-//   MODE SIGNAL: c2r, write x to out (pixel layout).
-//   MODE SIM: c2r, out = (w > 0) ? x + aux : 0 (aux = noise).
-//   MODE RFFT: r2c of the pixel rows of aux (a white field), store to scratch.
-// ---------------------------------------------------------------------------
-template <typename T, int MODE>
-__device__ __forceinline__ void k_row_body(WfGeo g, void* scratch_, const void* d_, const void* w_,
-                                           const void* aux_, void* out_, double* part, const void* tw_) {
+template <typename T>
+__device__ __forceinline__ void k_row_body(WfGeo g, void* scratch_, const void* w_, double* part, const void* tw_) {
   extern __shared__ __align__(16) unsigned char wf_smem[];
   V2<T>* s_tw = (V2<T>*)wf_smem;   // roots of unity (real-FFT pre/post twiddles)
   V2<T>* s_pt = s_tw + WF_NT;       // pass table of length nx/2
@@ -538,11 +417,7 @@ __device__ __forceinline__ void k_row_body(WfGeo g, void* scratch_, const void* 
   const int lgNTn = WF_LOG2_NT - g.lgnx;  // table stride of the nx-th roots
   double acc = 0.0;
 
-  if constexpr (MODE == WF_ROW_RFFT) {
-    const V2<T>* z = (const V2<T>*)((const T*)aux_ + (size_t)b * npix + (size_t)row0 * nx);
-    wf_g2s<T>(buf, z, tot);
-    __syncthreads();
-  } else {
+  {
     wf_g2s<T>(buf, sc, tot);
     __syncthreads();
     // c2r pre-processing: Z[k] = (X[k] + conj X[h-k]) + i w^k (X[k] - conj X[h-k]),
@@ -566,29 +441,15 @@ __device__ __forceinline__ void k_row_body(WfGeo g, void* scratch_, const void* 
     __syncthreads();
     fft_smem<T, +1, WF_EMAX>(buf, lgh, RB, h, 1, s_pt);
     // pixel stage: buf[t][m] holds pixels (2m, 2m+1) of row row0 + t
-    const V2<T>* dv = (const V2<T>*)((const T*)d_ + (size_t)b * npix + (size_t)row0 * nx);
     const V2<T>* wv = (const V2<T>*)((const T*)w_ + (size_t)b * npix + (size_t)row0 * nx);
-    if constexpr (MODE == WF_ROW_SIGNAL) {
-      V2<T>* ov = (V2<T>*)((T*)out_ + (size_t)b * npix + (size_t)row0 * nx);
-      wf_s2g<T>(ov, buf, tot);
-      return;
-    } else if constexpr (MODE == WF_ROW_SIM) {
-      V2<T>* ov = (V2<T>*)((T*)out_ + (size_t)b * npix + (size_t)row0 * nx);
-      const V2<T>* nz = (const V2<T>*)((const T*)aux_ + (size_t)b * npix + (size_t)row0 * nx);
-      for (int e = threadIdx.x; e < tot; e += blockDim.x) {
-        const V2<T> x = buf[wf_sw<T>(e)], w = wv[e], q = nz[e];
-        ov[e] = mk<T>(w.x > (T)0 ? x.x + q.x : (T)0, w.y > (T)0 ? x.y + q.y : (T)0);
-      }
-      return;
-    } else {
+    {
       float accf = 0.f;
-      V2<T> wl[WF_EMAX], dl[WF_EMAX];
+      V2<T> wl[WF_EMAX];
 #pragma unroll
       for (int i = 0; i < WF_EMAX; ++i) {
         const int e = threadIdx.x + i * WF_THREADS;
         if (e < tot) {
           wl[i] = wv[e];
-          if constexpr (MODE == WF_ROW_DATA) dl[i] = dv[e];
         }
       }
 #pragma unroll
@@ -596,9 +457,7 @@ __device__ __forceinline__ void k_row_body(WfGeo g, void* scratch_, const void* 
         const int e = threadIdx.x + i * WF_THREADS;
         if (e < tot) {
           const V2<T> x = buf[wf_sw<T>(e)], w = wl[i];
-          V2<T> r;
-          if constexpr (MODE == WF_ROW_DATA) r = mk<T>(dl[i].x - x.x, dl[i].y - x.y);
-          else r = mk<T>(-x.x, -x.y);
+          const V2<T> r = mk<T>(-x.x, -x.y);
           const V2<T> wr = mk<T>(w.x * r.x, w.y * r.y);
           if constexpr (sizeof(T) == 4) accf += r.x * wr.x + r.y * wr.y;
           else acc += (double)(r.x * wr.x) + (double)(r.y * wr.y);
@@ -631,17 +490,8 @@ __device__ __forceinline__ void k_row_body(WfGeo g, void* scratch_, const void* 
   }
   __syncthreads();
   wf_s2g<T>(sc, buf, tot);
-  if constexpr (MODE == WF_ROW_DATA || MODE == WF_ROW_NODATA) {
-    const double s = wf_block_sum(acc);
-    if (threadIdx.x == 0) part[((size_t)b * WF_NSLOT + WF_SLOT_DATA) * g.maxblk + blockIdx.x] = s;
-  }
-}
-
-template <typename T, int MODE>
-__global__ void __launch_bounds__(WF_THREADS, WF_MINB(T))
-k_row(WfGeo g, void* scratch_, const void* d_, const void* w_, const void* aux_, void* out_,
-      double* part, const void* tw_) {
-  k_row_body<T, MODE>(g, scratch_, d_, w_, aux_, out_, part, tw_);
+  const double s = wf_block_sum(acc);
+  if (threadIdx.x == 0) part[((size_t)b * WF_NSLOT + WF_SLOT_DATA) * g.maxblk + blockIdx.x] = s;
 }
 
 // chi2[b] = sum of the prior and data partial sums, in a fixed order.

@@ -26,96 +26,24 @@ template <typename K> inline cudaError_t ensure_smem(K kernel, size_t bytes, int
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (dev < 32 && (*done_mask >> dev) & 1) return cudaSuccess;
-  e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wf_pp_smem<double>());
+  e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
   if (e == cudaSuccess && dev < 32) *done_mask |= 1 << dev;
-  (void)bytes;
   return e;
 }
 
-// Resident blocks of a persistent kernel: SMs x blocks per SM (cached per device).
-template <typename K>
-inline cudaError_t persistent_grid(K k, size_t smem, int* occ, int* nsm, int* grid) {
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  const int di = dev & 31;
-  if (!occ[di]) {
-    int o = 0, ns = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, k, WF_THREADS, smem);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&ns, cudaDevAttrMultiProcessorCount, dev);
-    if (e != cudaSuccess) return e;
-    occ[di] = o > 0 ? o : 1;
-    nsm[di] = ns;
+// f<N>() of a register-resident length.
+template <class F> inline cudaError_t rg_length(int n, F&& f) {
+  switch (n) {
+    case 8: return f(std::integral_constant<int, 8>());
+    case 16: return f(std::integral_constant<int, 16>());
+    case 32: return f(std::integral_constant<int, 32>());
+    case 64: return f(std::integral_constant<int, 64>());
+    case 128: return f(std::integral_constant<int, 128>());
+    case 256: return f(std::integral_constant<int, 256>());
+    case 512: return f(std::integral_constant<int, 512>());
+    case 1024: return f(std::integral_constant<int, 1024>());
   }
-  *grid = occ[di] * nsm[di];
-  return cudaSuccess;
-}
-
-// Grid of a persistent launch over nitems work items: the resident blocks, at
-// most nitems (the items loop inside the kernel, so any grid is correct).
-template <typename K>
-inline cudaError_t items_grid(K k, size_t smem, int nitems, int* occ, int* nsm, int* grid) {
-  cudaError_t e = persistent_grid(k, smem, occ, nsm, grid);
-  if (e == cudaSuccess && *grid > nitems) *grid = nitems;
-  return e;
-}
-
-template <typename T, int C, int IN, int PLAN>
-cudaError_t col_inv_r(const WfGeo& g, const WfBufs& b, const void* src, cudaStream_t st) {
-  static int done = 0;
-  if constexpr (WF_FFT_PP && WF_COLINV_QUEUE) {
-    if (b.ticket) {
-      static int occq[32] = {0}, nsmq[32] = {0}, doneq = 0;
-      auto k = k_col_inv_pp_q<T, C, IN, PLAN>;
-      const size_t sm = wf_pp_smem<T>();
-      cudaError_t e = ensure_smem(k, sm, &doneq);
-      int grid = 0;
-      if (e == cudaSuccess) e = items_grid(k, sm, g.ntile * b.B, occq, nsmq, &grid);
-      if (e == cudaSuccess) e = cudaMemsetAsync(b.ticket, 0, sizeof(int), st);
-      if (e != cudaSuccess) return e;
-      k<<<grid, WF_THREADS, sm, st>>>(g, src, (const T*)b.sp, b.sp_stride, b.scratch, b.tw, b.B, b.ticket);
-      return cudaGetLastError();
-    }
-  }
-  if constexpr (WF_FFT_PP) {
-    static int occ[32] = {0}, nsm[32] = {0};
-    auto k = k_col_inv_pp_pers<T, C, IN, PLAN>;
-    const size_t sm = wf_pp_smem<T>();
-    cudaError_t e = ensure_smem(k, sm, &done);
-    int grid = 0;
-    if (e == cudaSuccess) e = items_grid(k, sm, g.ntile * b.B, occ, nsm, &grid);
-    if (e != cudaSuccess) return e;
-    k<<<grid, WF_THREADS, sm, st>>>(g, src, (const T*)b.sp, b.sp_stride, b.scratch, b.tw, b.B);
-    return cudaGetLastError();
-  } else {
-    auto k = k_col_inv<T, C, IN>;
-    const size_t sm = col_smem<T>(g);
-    cudaError_t e = ensure_smem(k, sm, &done);
-    if (e != cudaSuccess) return e;
-    k<<<dim3(g.ntile, b.B), WF_THREADS, sm, st>>>(g, src, (const T*)b.sp, b.sp_stride, b.scratch, b.tw);
-    return cudaGetLastError();
-  }
-}
-
-template <typename T, int C, int IN>
-cudaError_t col_inv(const WfGeo& g, const WfBufs& b, const void* src, cudaStream_t st) {
-  switch (wf_plan_eff(g.lgn, g.col_plan)) {
-    case 1: return col_inv_r<T, C, IN, 1>(g, b, src, st);
-    case 2: return col_inv_r<T, C, IN, 2>(g, b, src, st);
-    default: return col_inv_r<T, C, IN, 0>(g, b, src, st);
-  }
-}
-
-template <typename T, int C, int IN>
-cudaError_t col_fwd(const WfGeo& g, const WfBufs& b, const void* src, void* dst, cudaStream_t st) {
-  static int done = 0;
-  auto k = k_col_fwd<T, C, IN>;
-  const size_t sm = col_smem<T>(g);
-  cudaError_t e = ensure_smem(k, sm, &done);
-  if (e != cudaSuccess) return e;
-  k<<<dim3(g.ntile, b.B), WF_THREADS, sm, st>>>(g, src, (const T*)b.sp, b.sp_stride, b.scratch, dst,
-                                                b.part, b.tw);
-  return cudaGetLastError();
+  return cudaErrorInvalidValue;
 }
 
 // Deterministic band sums of standard-layout spectra (k_band_reduce, then
@@ -137,73 +65,17 @@ cudaError_t band_sums(const WfGeo& g, int B, const void* s, const void* grad, co
   return cudaGetLastError();
 }
 
-template <typename T, int C>
-cudaError_t col_sim(const WfGeo& g, const WfBufs& b, cudaStream_t st) {
-  static int done = 0;
-  auto k = k_col_sim<T, C>;
-  const size_t sm = col_smem<T>(g);
-  cudaError_t e = ensure_smem(k, sm, &done);
-  if (e != cudaSuccess) return e;
-  k<<<dim3(g.ntile, b.B), WF_THREADS, sm, st>>>(g, (const T*)b.sp, b.sp_stride, b.scratch, b.tw);
-  return cudaGetLastError();
-}
-
-template <typename T, int MODE>
-cudaError_t row(const WfGeo& g, const WfBufs& b, const void* aux, void* out, cudaStream_t st) {
-  static int done = 0;
-  if constexpr (WF_FFT_PP && (MODE == WF_ROW_DATA || MODE == WF_ROW_NODATA)) {
-    static int done_pp[WF_NPLAN] = {0};
-    const int pl = wf_plan_eff(g.lgh, g.row_plan);
-    auto k = pl == 1 ? k_row_pp<T, MODE, 1> : pl == 2 ? k_row_pp<T, MODE, 2> : k_row_pp<T, MODE, 0>;
-    const size_t sm = wf_pp_smem<T>();
-    cudaError_t e = ensure_smem(k, sm, &done_pp[pl]);
-    if (e != cudaSuccess) return e;
-    k<<<dim3(g.nrb, b.B), WF_THREADS, sm, st>>>(g, b.scratch, b.d, b.w, b.part, b.tw);
-    return cudaGetLastError();
-  }
-  auto k = k_row<T, MODE>;
-  const size_t sm = row_smem<T>(g);
-  cudaError_t e = ensure_smem(k, sm, &done);
-  if (e != cudaSuccess) return e;
-  k<<<dim3(g.nrb, b.B), WF_THREADS, sm, st>>>(g, b.scratch, b.d, b.w, aux, out, b.part, b.tw);
-  return cudaGetLastError();
-}
-
 template <typename T>
-cudaError_t row_any(int mode, const WfGeo& g, const WfBufs& b, const void* aux, void* out,
-                    cudaStream_t st) {
-  switch (mode) {
-    case WF_ROW_DATA: return row<T, WF_ROW_DATA>(g, b, aux, out, st);
-    case WF_ROW_NODATA: return row<T, WF_ROW_NODATA>(g, b, aux, out, st);
-    case WF_ROW_SIGNAL: return row<T, WF_ROW_SIGNAL>(g, b, aux, out, st);
-    case WF_ROW_SIM: return row<T, WF_ROW_SIM>(g, b, aux, out, st);
-    case WF_ROW_RFFT: return row<T, WF_ROW_RFFT>(g, b, aux, out, st);
-  }
-  return cudaErrorInvalidValue;
+cudaError_t row(int mode, const WfGeo& g, const WfBufs& b, const void* aux, void* out, cudaStream_t st) {
+  return rg_length(g.nx, [&](auto n) { return wf_reg_row<T, n()>(g, b, mode, aux, out, st); });
 }
-
 template <typename T>
-cudaError_t col_inv_any(const WfGeo& g, const WfBufs& b, int in, const void* src, cudaStream_t st) {
-  if (g.C == 1) return in == WF_IN_PK ? col_inv<T, 1, WF_IN_PK>(g, b, src, st) : col_inv<T, 1, WF_IN_STD>(g, b, src, st);
-  return in == WF_IN_PK ? col_inv<T, 2, WF_IN_PK>(g, b, src, st) : col_inv<T, 2, WF_IN_STD>(g, b, src, st);
+cudaError_t col_inv(const WfGeo& g, const WfBufs& b, int in, const void* src, cudaStream_t st) {
+  return rg_length(g.n, [&](auto n) { return wf_reg_colinv<T, n()>(g, b, in, src, st); });
 }
-
 template <typename T>
-cudaError_t col_fwd_any(const WfGeo& g, const WfBufs& b, int in, const void* src, void* dst,
-                        cudaStream_t st) {
-  if (g.C == 1)
-    return in == WF_IN_PK ? col_fwd<T, 1, WF_IN_PK>(g, b, src, dst, st) : col_fwd<T, 1, WF_IN_STD>(g, b, src, dst, st);
-  return in == WF_IN_PK ? col_fwd<T, 2, WF_IN_PK>(g, b, src, dst, st) : col_fwd<T, 2, WF_IN_STD>(g, b, src, dst, st);
-}
-
-template <typename K> inline cudaError_t ensure_smem_n(K kernel, size_t bytes, int* done_mask) {
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  if (dev < 32 && (*done_mask >> dev) & 1) return cudaSuccess;
-  e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-  if (e == cudaSuccess && dev < 32) *done_mask |= 1 << dev;
-  return e;
+cudaError_t col_fwd(const WfGeo& g, const WfBufs& b, int in, const void* src, void* dst, cudaStream_t st) {
+  return rg_length(g.n, [&](auto n) { return wf_reg_colfwd<T, n()>(g, b, in, src, dst, st); });
 }
 
 // cuTensorMapEncodeTiled, fetched from the driver once (no link to libcuda).
@@ -230,7 +102,7 @@ cudaError_t lb_colinv_tma(const WfGeo& g, const WfBufs& b, const WfLbBufs& lb, c
   static int occ[32] = {0}, nsm[32] = {0};
   auto k = k_lb_colinv_tma<T, C, PLAN>;
   const size_t sm = wf_colinv_tma_smem<T>();
-  cudaError_t e = ensure_smem_n(k, sm, &done);
+  cudaError_t e = ensure_smem(k, sm, &done);
   if (e != cudaSuccess) return e;
   int dev = 0;
   e = cudaGetDevice(&dev);
@@ -264,29 +136,26 @@ cudaError_t lb_colinv_tma(const WfGeo& g, const WfBufs& b, const WfLbBufs& lb, c
 }
 
 
-template <typename T, int C, int KIND, int PLAN>
+template <typename T, int C>
 cudaError_t lb_colinv_tile(const WfGeo& g, const WfBufs& b, const WfLbBufs& lb, cudaStream_t st) {
   static int done = 0;
-  auto k = k_lb_colinv<T, C, KIND, PLAN>;
-  const size_t sm = KIND == WF_COLINV_PP_K ? wf_pp_smem<T>() : col_smem<T>(g);
-  cudaError_t e = ensure_smem(k, sm, &done);
+  auto k = k_lb_colinv<T, C>;
+  const size_t sm = col_smem<T>(g);
+  cudaError_t e = ensure_smem(k, (WF_NT + (size_t)WF_TILE) * sizeof(V2<T>), &done);  // the widest tile
   if (e != cudaSuccess) return e;
   k<<<dim3(g.ntile, b.B), WF_THREADS, sm, st>>>(g, (const T*)b.sp, b.sp_stride, b.scratch, b.tw, lb);
   return cudaGetLastError();
 }
 
 // The variant in g.colinv_kind (the TMA form needs the driver's tensor-map
-// encoder; without it the ping-pong form runs).
+// encoder; without it the in-place form runs its tiles).
 template <typename T, int C>
 cudaError_t lb_colinv(const WfGeo& g, const WfBufs& b, const WfLbBufs& lb, cudaStream_t st) {
   const int pl = wf_plan_eff(g.lgn, g.col_plan);
   if (g.colinv_kind == WF_COLINV_TMA_K && wf_encode_fn())
     return pl == 1 ? lb_colinv_tma<T, C, 1>(g, b, lb, st)
            : pl == 2 ? lb_colinv_tma<T, C, 2>(g, b, lb, st) : lb_colinv_tma<T, C, 0>(g, b, lb, st);
-  if (g.colinv_kind == WF_COLINV_INPLACE_K) return lb_colinv_tile<T, C, WF_COLINV_INPLACE_K, 0>(g, b, lb, st);
-  return pl == 1 ? lb_colinv_tile<T, C, WF_COLINV_PP_K, 1>(g, b, lb, st)
-         : pl == 2 ? lb_colinv_tile<T, C, WF_COLINV_PP_K, 2>(g, b, lb, st)
-                   : lb_colinv_tile<T, C, WF_COLINV_PP_K, 0>(g, b, lb, st);
+  return lb_colinv_tile<T, C>(g, b, lb, st);
 }
 
 template <typename T, int C>
@@ -294,7 +163,7 @@ cudaError_t lb_colfwd(const WfGeo& g, const WfBufs& b, const WfLbBufs& lb, cudaS
   static int done = 0;
   auto k = k_lb_colfwd<T, C>;
   const size_t sm = col_smem<T>(g);
-  cudaError_t e = ensure_smem(k, sm, &done);
+  cudaError_t e = ensure_smem(k, (WF_NT + (size_t)WF_TILE) * sizeof(V2<T>), &done);  // the widest tile
   if (e != cudaSuccess) return e;
   k<<<dim3(g.ntile, b.B), WF_THREADS, sm, st>>>(g, (const T*)b.sp, b.sp_stride, b.scratch, b.tw, lb, b.part);
   return cudaGetLastError();
@@ -342,9 +211,9 @@ inline int grid1d(size_t total, int cap) {
   template <typename T>
   cudaError_t wf_launch_eval(const WfGeo& g, const WfBufs& b, int row_mode, int in_layout,
                                 const void* src, void* dst, double* chi2, cudaStream_t st) {
-    cudaError_t e = wfimpl::col_inv_any<T>(g, b, in_layout, src, st);
-    if (e == cudaSuccess) e = wfimpl::row_any<T>(row_mode, g, b, nullptr, nullptr, st);
-    if (e == cudaSuccess) e = wfimpl::col_fwd_any<T>(g, b, in_layout, src, dst, st);
+    cudaError_t e = wfimpl::col_inv<T>(g, b, in_layout, src, st);
+    if (e == cudaSuccess) e = wfimpl::row<T>(row_mode, g, b, nullptr, nullptr, st);
+    if (e == cudaSuccess) e = wfimpl::col_fwd<T>(g, b, in_layout, src, dst, st);
     if (e == cudaSuccess && chi2) {
       k_finalize_chi2<<<b.B, WF_THREADS, 0, st>>>(b.part, g.maxblk, g.ntile,
                                                   row_mode == WF_ROW_DATA ? g.nrb : 0, chi2);
@@ -355,17 +224,16 @@ inline int grid1d(size_t total, int cap) {
   template <typename T>
   cudaError_t wf_launch_signal(const WfGeo& g, const WfBufs& b, int in_layout, const void* src,
                                   void* xout, cudaStream_t st) {
-    cudaError_t e = wfimpl::col_inv_any<T>(g, b, in_layout, src, st);
-    if (e == cudaSuccess) e = wfimpl::row_any<T>(WF_ROW_SIGNAL, g, b, nullptr, xout, st);
+    cudaError_t e = wfimpl::col_inv<T>(g, b, in_layout, src, st);
+    if (e == cudaSuccess) e = wfimpl::row<T>(WF_ROW_SIGNAL, g, b, nullptr, xout, st);
     return e;
   }
   template <typename T>
   cudaError_t wf_launch_simulate(const WfGeo& g, const WfBufs& b, const void* z,
                                     const void* noise, void* dout, cudaStream_t st) {
-    cudaError_t e = wfimpl::row_any<T>(WF_ROW_RFFT, g, b, z, nullptr, st);
-    if (e == cudaSuccess)
-      e = g.C == 1 ? wfimpl::col_sim<T, 1>(g, b, st) : wfimpl::col_sim<T, 2>(g, b, st);
-    if (e == cudaSuccess) e = wfimpl::row_any<T>(WF_ROW_SIM, g, b, noise, dout, st);
+    cudaError_t e = wfimpl::row<T>(WF_ROW_RFFT, g, b, z, nullptr, st);
+    if (e == cudaSuccess) e = wfimpl::rg_length(g.n, [&](auto n) { return wf_reg_colsim<T, n()>(g, b, st); });
+    if (e == cudaSuccess) e = wfimpl::row<T>(WF_ROW_SIM, g, b, noise, dout, st);
     return e;
   }
   template <typename T>
@@ -410,7 +278,7 @@ cudaError_t wf_launch_lb_comb(const WfGeo& g, const WfBufs& b, const WfLbBufs& l
   static int done = 0;
   auto k = k_lb_comb<T>;
   const size_t sm = wf_comb_smem<T>(lb.m);
-  cudaError_t e = wfimpl::ensure_smem_n(k, wf_comb_smem<T>(WF_MAXM), &done);
+  cudaError_t e = wfimpl::ensure_smem(k, wf_comb_smem<T>(WF_MAXM), &done);
   if (e != cudaSuccess) return e;
   k<<<dim3(g.ncomb, b.B), WF_COMB_THREADS, sm, st>>>(g, lb, b.part, mode);
   return cudaGetLastError();
@@ -420,44 +288,37 @@ cudaError_t wf_launch_lb_qdots(const WfGeo& g, const WfBufs& b, const WfLbBufs& 
   static int done = 0;
   auto k = k_lb_qdots<T>;
   const size_t sm = wf_comb_smem<T>(lb.m);
-  cudaError_t e = wfimpl::ensure_smem_n(k, wf_comb_smem<T>(WF_MAXM), &done);
+  cudaError_t e = wfimpl::ensure_smem(k, wf_comb_smem<T>(WF_MAXM), &done);
   if (e != cudaSuccess) return e;
   k<<<dim3(g.ncomb, b.B), WF_COMB_THREADS, sm, st>>>(g, lb, b.part);
   return cudaGetLastError();
 }
 template <typename T>
 cudaError_t wf_launch_lb_colinv(const WfGeo& g, const WfBufs& b, const WfLbBufs& lb, cudaStream_t st) {
+  if (g.colinv_kind == WF_COLINV_REG_K) return wfimpl::rg_length(g.n, [&](auto n) { return wf_reg_lb_colinv<T, n()>(g, b, lb, st); });
   return g.C == 1 ? wfimpl::lb_colinv<T, 1>(g, b, lb, st) : wfimpl::lb_colinv<T, 2>(g, b, lb, st);
 }
 template <typename T>
 cudaError_t wf_launch_lb_colfwd(const WfGeo& g, const WfBufs& b, const WfLbBufs& lb, cudaStream_t st) {
+  if (g.colinv_kind == WF_COLINV_REG_K) return wfimpl::rg_length(g.n, [&](auto n) { return wf_reg_lb_colfwd<T, n()>(g, b, lb, st); });
   return g.C == 1 ? wfimpl::lb_colfwd<T, 1>(g, b, lb, st) : wfimpl::lb_colfwd<T, 2>(g, b, lb, st);
 }
-namespace wfimpl {
-template <typename T, int KIND, int PLAN>
-cudaError_t lb_row(const WfGeo& g, const WfBufs& b, const WfLbBufs& lb, cudaStream_t st) {
+template <typename T>
+cudaError_t wf_launch_lb_row(const WfGeo& g, const WfBufs& b, const WfLbBufs& lb, cudaStream_t st) {
+  if (g.row_kind == WF_ROW_REG_K) return wfimpl::rg_length(g.nx, [&](auto n) { return wf_reg_lb_row<T, n()>(g, b, lb, st); });
   static int done = 0;
-  auto k = k_lb_row<T, KIND, PLAN>;
-  const size_t sm = KIND == WF_ROW_PP_K ? wf_pp_smem<T>() : row_smem<T>(g);
-  cudaError_t e = ensure_smem(k, sm, &done);
+  auto k = k_lb_row<T>;
+  const size_t sm = wfimpl::row_smem<T>(g);
+  cudaError_t e = wfimpl::ensure_smem(k, (2 * WF_NT + (size_t)WF_TILE) * sizeof(V2<T>), &done);
   if (e != cudaSuccess) return e;
   k<<<dim3(g.nrb, b.B), WF_THREADS, sm, st>>>(g, b.scratch, b.w, b.part, b.tw, lb.st);
   return cudaGetLastError();
 }
-}  // namespace wfimpl
-template <typename T>
-cudaError_t wf_launch_lb_row(const WfGeo& g, const WfBufs& b, const WfLbBufs& lb, cudaStream_t st) {
-  if (g.row_kind == WF_ROW_INPLACE_K) return wfimpl::lb_row<T, WF_ROW_INPLACE_K, 0>(g, b, lb, st);
-  const int pl = wf_plan_eff(g.lgh, g.row_plan);
-  return pl == 1 ? wfimpl::lb_row<T, WF_ROW_PP_K, 1>(g, b, lb, st)
-         : pl == 2 ? wfimpl::lb_row<T, WF_ROW_PP_K, 2>(g, b, lb, st)
-                   : wfimpl::lb_row<T, WF_ROW_PP_K, 0>(g, b, lb, st);
-}
 template <typename T>
 cudaError_t wf_launch_eval_pk(const WfGeo& g, const WfBufs& b, const void* src, void* dst, cudaStream_t st) {
-  cudaError_t e = wfimpl::col_inv_any<T>(g, b, WF_IN_PK, src, st);
-  if (e == cudaSuccess) e = wfimpl::row_any<T>(WF_ROW_DATA, g, b, nullptr, nullptr, st);
-  if (e == cudaSuccess) e = wfimpl::col_fwd_any<T>(g, b, WF_IN_PK, src, dst, st);
+  cudaError_t e = wfimpl::col_inv<T>(g, b, WF_IN_PK, src, st);
+  if (e == cudaSuccess) e = wfimpl::row<T>(WF_ROW_DATA, g, b, nullptr, nullptr, st);
+  if (e == cudaSuccess) e = wfimpl::col_fwd<T>(g, b, WF_IN_PK, src, dst, st);
   return e;
 }
 

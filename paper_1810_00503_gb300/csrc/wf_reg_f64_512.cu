@@ -1,0 +1,4 @@
+// Register-resident stages of length 512, FP64.
+#include "wf_reg_impl.cuh"
+WF_RG_INSTANTIATE(double, 512)
+WF_DBG_READER(reg_f64_512)

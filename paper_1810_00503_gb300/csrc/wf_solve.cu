@@ -601,12 +601,14 @@ static cudaError_t refresh(const wf_problem* p, const WfBufs& b, const WfLbBufs&
                            WfSolver* S, cudaStream_t st) {
   cudaError_t e = cudaSuccess;
   if (!init) e = wf_launch_lb_comb<T>(p->g, b, lb, WF_LB1_MATERIALIZE, st);
-  if (e == cudaSuccess) e = wf_launch_eval_pk<T>(p->g, b, lb.s, lb.g, st);
+  if (e == cudaSuccess) e = wf_launch_eval_pk<T>(p->gp, b, lb.s, lb.g, st);
   if (e == cudaSuccess) e = wf_launch_lb_comb<T>(p->g, b, lb, WF_LB1_DOTS, st);
   if (e == cudaSuccess) e = cudaMemsetAsync(S->nact, 0, sizeof(int), st);
   if (e == cudaSuccess) {
     A.phase = WF_PH_REFRESH;
     A.init = init;
+    A.ntile = p->gp.ntile;
+    A.nrb = p->gp.nrb;
     k_lb_scalar<<<(p->count + WF_SW - 1) / WF_SW, 32 * WF_SW, 0, st>>>(lb.st, b.part, A, p->count, S->nact);
     e = cudaGetLastError();
   }
@@ -637,7 +639,10 @@ static bool variant_valid(int v) {
             d = v % 10;
   auto div_ok = [](int x) { return x == 1 || x == 2 || x == 4; };
   return v >= 1000 && f < WF_NPLAN && e < WF_NPLAN && a >= WF_COLINV_TMA_K && a <= WF_COLINV_INPLACE_K &&
-         b >= WF_ROW_PP_K && b <= WF_ROW_INPLACE_K && div_ok(c) && div_ok(d);
+         b >= WF_ROW_REG_K && b <= WF_ROW_INPLACE_K && div_ok(c) && div_ok(d);
+}
+static WfGeo default_geo(const wf_problem* p) {
+  return wf_make_geo(p->n, p->nx, p->C, p->count);
 }
 static WfGeo variant_geo(const WfGeo& base, int v) {
   return wf_geo_variant(base, (v / 1000) % 10, (v / 100) % 10, (v / 10) % 10, v % 10, v / 100000,
@@ -683,14 +688,13 @@ template <typename T>
 static wf_status choose_variant(wf_problem* p, WfSolver* S, cudaStream_t st) {
   const wf_opts* o = &S->o;
   const bool shared = S->shared_tune != 0;
-  const WfGeo base = shared ? variant_geo(wf_make_geo(p->n, p->nx, p->C, p->count), WF_MULTI_VARIANT)
-                            : wf_make_geo(p->n, p->nx, p->C, p->count);
+  const WfGeo base = shared ? variant_geo(default_geo(p), WF_MULTI_VARIANT) : default_geo(p);
   if (o->fft_variant) {
     p->g = variant_geo(base, o->fft_variant);
     return WF_OK;
   }
-  if (!o->autotune || o->inject_timeout_map > 0) {  // the injected wait lives in the TMA-fed stage
-    p->g = base;
+  if (!o->autotune || o->inject_timeout_map > 0) {
+    p->g = o->inject_timeout_map > 0 ? variant_geo(base, WF_TMA_VARIANT) : base;  // the injected wait lives there
     return WF_OK;
   }
   const int m = S->o.lbfgs_m;
@@ -746,15 +750,15 @@ static wf_status choose_variant(wf_problem* p, WfSolver* S, cudaStream_t st) {
     return ms;
   };
   // column choices (inverse and forward column stage together), then the row
-  // choices with the column choice fixed; radix plans only for the ping-pong
-  // passes, and only those that differ at this length
+  // choices with the column choice fixed; radix plans only for the TMA-fed
+  // stage, and only those that differ at this length
   WfGeo best = base;
   float best_ms = INFINITY;
   const int divs[3] = {1, 2, 4};
   for (int ck = WF_COLINV_TMA_K; ck <= WF_COLINV_INPLACE_K; ++ck)
-    for (int cp = 0; cp < (ck == WF_COLINV_INPLACE_K ? 1 : WF_NPLAN); ++cp) {
+    for (int cp = 0; cp < (ck == WF_COLINV_TMA_K ? WF_NPLAN : 1); ++cp) {
       if (!plan_new(p->g.lgn, cp)) continue;
-      if (shared && (ck != base.colinv_kind || cp != base.col_plan)) continue;
+      if (shared && ck != base.colinv_kind) continue;
       int last_tc = -1;
       for (int di : divs) {
         const WfGeo g = wf_geo_variant(base, ck, base.row_kind, di, 1, cp, 0);
@@ -770,19 +774,17 @@ static wf_status choose_variant(wf_problem* p, WfSolver* S, cudaStream_t st) {
     }
   best_ms = INFINITY;
   WfGeo bestr = best;
-  for (int rk = WF_ROW_PP_K; rk <= WF_ROW_INPLACE_K; ++rk)
-    for (int rp = 0; rp < (rk == WF_ROW_INPLACE_K ? 1 : WF_NPLAN); ++rp) {
-      if (!plan_new(p->g.lgh, rp)) continue;
-      if (shared && (rk != base.row_kind || rp != base.row_plan)) continue;
-      int last_rb = -1;
-      for (int di : divs) {
-        const WfGeo g = wf_geo_variant(base, best.colinv_kind, rk, best.tc_div, di, best.col_plan, rp);
-        if (g.RB == last_rb) continue;
-        last_rb = g.RB;
-        const float ms = timed([&]() { return wf_launch_lb_row<T>(g, b, lb, st); });
-        if (ms < best_ms) { best_ms = ms; bestr = g; }
-      }
+  for (int rk = WF_ROW_REG_K; rk <= WF_ROW_INPLACE_K; ++rk) {
+    if (shared && rk != base.row_kind) continue;
+    int last_rb = -1;
+    for (int di : divs) {
+      const WfGeo g = wf_geo_variant(base, best.colinv_kind, rk, best.tc_div, di, best.col_plan, 0);
+      if (g.RB == last_rb) continue;
+      last_rb = g.RB;
+      const float ms = timed([&]() { return wf_launch_lb_row<T>(g, b, lb, st); });
+      if (ms < best_ms) { best_ms = ms; bestr = g; }
     }
+  }
   cudaStreamSynchronize(st);
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
@@ -1002,12 +1004,12 @@ static wf_status finish_impl(wf_problem* p, void* s_out, void* x_out, wf_solve_s
   WfBufs b = wf_bufs(p);
   WfLbBufs lb = lb_bufs<T>(S);
   WF_TRY(wf_launch_lb_comb<T>(p->g, b, lb, WF_LB1_MATERIALIZE, st));
-  WF_TRY(wf_launch_eval_pk<T>(p->g, b, lb.s, lb.g, st));
-  k_lb_final<<<(p->count + WF_SW - 1) / WF_SW, 32 * WF_SW, 0, st>>>(lb.st, b.part, p->g.ntile, p->g.nrb,
-                                                                    p->g.maxblk, p->count, S->stats_dev);
+  WF_TRY(wf_launch_eval_pk<T>(p->gp, b, lb.s, lb.g, st));
+  k_lb_final<<<(p->count + WF_SW - 1) / WF_SW, 32 * WF_SW, 0, st>>>(lb.st, b.part, p->gp.ntile, p->gp.nrb,
+                                                                    p->gp.maxblk, p->count, S->stats_dev);
   WF_TRY(cudaGetLastError());
   if (s_out) WF_TRY(wf_launch_unpack<T>(p->g, p->count, S->s, s_out, st));
-  if (x_out) WF_TRY(wf_launch_signal<T>(p->g, b, WF_IN_PK, S->s, x_out, st));
+  if (x_out) WF_TRY(wf_launch_signal<T>(p->gp, b, WF_IN_PK, S->s, x_out, st));
   WF_TRY(cudaMemcpyAsync(S->stats_host, S->stats_dev, sizeof(double) * 5 * p->count, cudaMemcpyDeviceToHost, st));
   WF_TRY(cudaEventRecord(S->ev_out, st));
   WF_TRY(cudaStreamWaitEvent(us, S->ev_out, 0));
@@ -1081,7 +1083,7 @@ static wf_status refined_impl(wf_problem* p, const wf_opts* o, double tol, int m
   // The FP64 operator of the outer evaluations: for a MIXED problem on exact
   // FP64 copies of the working-precision inputs (the problem the inner solves
   // see), always on the default tiles.
-  const WfGeo go = wf_make_geo(p->n, p->nx, p->C, p->count);
+  const WfGeo& go = p->gp;
   WfBufs bo = wf_bufs(p);
   if (mixed) {
     k_convert<float, double><<<wf_grid(per * B), 256, 0, st>>>((const float*)p->d, (double*)S->r_d64, per * B);
@@ -1237,7 +1239,7 @@ static wf_status check_opts(const wf_problem* p, const wf_opts* o) {
                    o->fft_variant);
   if (o->inject_timeout_map < 0 || o->inject_timeout_map > p->count)
     return wf_fail(WF_EINVAL, "inject_timeout_map = %d outside [0, %d]", o->inject_timeout_map, p->count);
-  if (o->inject_timeout_map > 0 && wf_make_geo(p->n, p->nx, p->C).colinv_kind != WF_COLINV_TMA_K)
+  if (o->inject_timeout_map > 0 && variant_geo(default_geo(p), WF_TMA_VARIANT).colinv_kind != WF_COLINV_TMA_K)
     return wf_fail(WF_EINVAL, "inject_timeout_map: %d x %d maps have no TMA-fed inverse column stage", p->n,
                    p->nx);
   if (o->line_search != WF_LS_EXACT && o->line_search != WF_LS_WOLFE)
@@ -1331,16 +1333,18 @@ static cudaError_t any_refresh(wf_problem* p, cudaStream_t st) {
                                  : refresh<float>(p, wf_bufs(p), lb_bufs<float>(S), S->A, 0, S, st);
 }
 
-// One L-BFGS iteration of several problems in shared launches (see
-// WfMultiArgs): the five kernels of iteration() plus the active counters'
-// reset and the scalar step, seven launches whatever the number of problems.
+// One L-BFGS iteration of several problems: the streaming kernels, the active
+// counters' reset and the scalar step in launches shared by all (see
+// WfMultiArgs), the FFT stages per problem.
 static_assert(WF_SW == 1, "the shared scalar launch takes one block per map");
 template <typename T>
 static cudaError_t multi_iteration(const WfMultiArgs& a, const WfMultiScalar& ms, cudaStream_t st) {
   cudaError_t e = wf_launch_multi_comb<T>(a, WF_LB1_FULL, st);
-  if (e == cudaSuccess) e = wf_launch_multi_colinv<T>(a, st);
-  if (e == cudaSuccess) e = wf_launch_multi_row<T>(a, st);
-  if (e == cudaSuccess) e = wf_launch_multi_colfwd<T>(a, st);
+  for (int q = 0; q < a.np && e == cudaSuccess; ++q) {
+    e = wf_launch_lb_colinv<T>(a.g[q], a.b[q], a.lb[q], st);
+    if (e == cudaSuccess) e = wf_launch_lb_row<T>(a.g[q], a.b[q], a.lb[q], st);
+    if (e == cudaSuccess) e = wf_launch_lb_colfwd<T>(a.g[q], a.b[q], a.lb[q], st);
+  }
   if (e == cudaSuccess) e = wf_launch_multi_qdots<T>(a, st);
   if (e == cudaSuccess) {
     k_multi_zero<<<1, 32, 0, st>>>(ms);
@@ -1356,9 +1360,9 @@ static cudaError_t multi_iteration(const WfMultiArgs& a, const WfMultiScalar& ms
 // Several problems (typically one per map shape of a heterogeneous batch)
 // solved as one batch.  Every problem is started on its own stream (first
 // gradient).  When the problems share the working type and C (and no FFT-stage
-// variant is forced), each iteration of the whole batch is seven shared
-// launches (multi_iteration), every problem on the ping-pong stages of
-// WF_MULTI_VARIANT with its own tuned tile widths; otherwise each problem is
+// variant is forced), an iteration of the whole batch shares its streaming and
+// scalar launches (multi_iteration), every problem on the register-resident
+// stages of WF_MULTI_VARIANT with its own tuned tile widths; otherwise each problem is
 // tuned freely and runs its own kernels, as a parallel branch per problem.  check_every iterations are
 // captured in one CUDA graph, so that each round is one graph launch for the
 // whole batch; the maps of every shape advance together and a problem whose
@@ -1599,7 +1603,7 @@ static wf_status import_impl(wf_problem* p, const WfStateHeader& hd, const char*
   cudaStream_t st = wf_capturable(us) ? us : S->stream;
   if (S->exec) { cudaGraphExecDestroy(S->exec); S->exec = nullptr; }
   S->work = st;
-  p->g = variant_geo(wf_make_geo(p->n, p->nx, p->C, p->count), hd.variant);
+  p->g = variant_geo(default_geo(p), hd.variant);
   rs = setup_args(p, S, &S->o);
   if (rs != WF_OK) return rs;
   size_t off_st, off_vec;

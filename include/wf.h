@@ -357,14 +357,13 @@ wf_status wf_solver_history(const wf_problem* p, double* out, int* counts);
  * shape of a heterogeneous batch (Sec. 2.2; the simulations of Sec. 2.5 need
  * not share a size).  Every problem is started on its own internal stream,
  * ordered after opts->stream (first gradient).  When 2 to 8 problems share
- * the precision and C and opts->fft_variant is 0, the streaming kernels and
- * the scalar step of each L-BFGS iteration are launches shared by the whole
- * batch: every launch covers the blocks of every problem's own grid, each
- * block running the single-problem kernel at its place in its problem's grid;
- * the FFT stages are launched per problem, every problem on the
- * register-resident stages with its own tile widths (tuned per shape when
- * opts->autotune, else the widest: variant 2111), so each map ends exactly
- * where its problem solved alone with the
+ * the precision and C and opts->fft_variant is 0, each L-BFGS iteration of
+ * the whole batch is one set of seven shared launches: every launch covers
+ * the blocks of every problem's own grid, each block running the
+ * single-problem kernel at its place in its problem's grid, every problem on
+ * the register-resident column and row stages with its own tile widths (tuned
+ * per shape when opts->autotune, else the widest: variant 2111), so each map
+ * ends exactly where its problem solved alone with the
  * variant its stats report ends.  Otherwise every problem is tuned and
  * runs its own kernels, a parallel branch per problem.  opts->check_every
  * iterations are captured in one CUDA graph, so that each round of the batch

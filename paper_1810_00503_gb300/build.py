@@ -20,6 +20,7 @@ LIB = os.path.join(HERE, "libwf.so")
 SOURCES = ["wf_api.cu", "wf_solve.cu", "wf_ops_f32.cu", "wf_ops_f64.cu", "wf_lbcol_f32.cu", "wf_lbcol_f64.cu",
            "wf_lbrow_f32.cu", "wf_lbrow_f64.cu", "wf_noalloc.cu", "wf_bandpower.cu", "wf_rng.cu", "wf_peak.cu",
            "wf_multi.cu", "wf_any.cu",
+           "wf_multi_f32_c1.cu", "wf_multi_f32_c2.cu", "wf_multi_f64_c1.cu", "wf_multi_f64_c2.cu",
            "wf_reg_f32_small.cu", "wf_reg_f32_256.cu", "wf_reg_f32_512.cu", "wf_reg_f32_1024.cu",
            "wf_reg_f64_small.cu", "wf_reg_f64_256.cu", "wf_reg_f64_512.cu", "wf_reg_f64_1024.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]

@@ -53,7 +53,7 @@ __device__ __forceinline__ long long wf_chk(long long i, long long lim, int line
 #endif
 #define WF_DBG_TUS(X) X(ops_f32) X(ops_f64) X(lbcol_f32) X(lbcol_f64) X(lbrow_f32) X(lbrow_f64) X(solve) X(noalloc) X(bandpower) X(multi) X(any) \
   X(reg_f32_small) X(reg_f32_256) X(reg_f32_512) X(reg_f32_1024) X(reg_f64_small) X(reg_f64_256) X(reg_f64_512) \
-  X(reg_f64_1024)
+  X(reg_f64_1024) X(multi_f32_c1) X(multi_f32_c2) X(multi_f64_c1) X(multi_f64_c2)
 #define WF_DBG_DECL(name) cudaError_t wf_dbg_read_##name(unsigned long long* out, int reset);
 WF_DBG_TUS(WF_DBG_DECL)
 
@@ -318,9 +318,8 @@ struct WfLbBufs {
   int inject_map;   // map whose tile copies are never issued (-1: none), see wf_opts
   long long spin_limit;  // bound of device waits, SM cycles
 };
-// Streaming launches shared by several problems (wf_map_solve_many: one problem
-// per map shape of a heterogeneous batch; the FFT stages, whose code differs by
-// length, are launched per problem).  Every problem keeps its own geometry,
+// Launches shared by several problems (wf_map_solve_many: one problem per map
+// shape of a heterogeneous batch).  Every problem keeps its own geometry,
 // buffers and L-BFGS state; a shared launch covers the blocks of every
 // problem's own grid, problem q's at blocks start[q] .. start[q+1] - 1, and
 // each block runs the single-problem kernel body at its coordinates in its
@@ -339,6 +338,9 @@ struct WfMultiArgs {
 #define WF_TMA_VARIANT 1111  // the TMA-fed inverse column stage, widest tiles
 template <typename T>
 cudaError_t wf_launch_multi_comb(const WfMultiArgs& a, int mode, cudaStream_t st);
+// stage: 0 inverse column, 1 row, 2 forward column.
+template <typename T, int C>
+cudaError_t wf_launch_multi_fft(const WfMultiArgs& a, int stage, cudaStream_t st);
 template <typename T>
 cudaError_t wf_launch_multi_qdots(const WfMultiArgs& a, cudaStream_t st);
 

@@ -1,0 +1,4 @@
+// Shared FFT-stage launches, FP32, 2 channels.
+#include "wf_multi_fft.cuh"
+template cudaError_t wf_launch_multi_fft<float, 2>(const WfMultiArgs&, int, cudaStream_t);
+WF_DBG_READER(multi_f32_c2)

@@ -1,0 +1,4 @@
+// Shared FFT-stage launches, FP64, 2 channels.
+#include "wf_multi_fft.cuh"
+template cudaError_t wf_launch_multi_fft<double, 2>(const WfMultiArgs&, int, cudaStream_t);
+WF_DBG_READER(multi_f64_c2)

@@ -1,0 +1,89 @@
+// FFT stages of the L-BFGS iteration in launches shared by several problems
+// (wf_map_solve_many), for one working type and channel count: every block finds
+// its problem and runs the register-resident stage of that problem's length and
+// tile width, so a batch of any mix of shapes takes three launches (a branch per
+// problem instead, captured in the batch's graph, took 1.4 times as long on
+// batches of few small maps: capturing and instantiating a node costs more than
+// its kernel).  Blocks are as large as the widest stage's; threads a narrower one
+// has no use for leave at once.
+#pragma once
+#include "wf_multi.cuh"
+#include "wf_reg.cuh"
+
+// f<N>() of length n.
+template <class F> __device__ __forceinline__ void wf_rg_switch(int n, F&& f) {
+  switch (n) {
+    case 8: f(std::integral_constant<int, 8>()); break;
+    case 16: f(std::integral_constant<int, 16>()); break;
+    case 32: f(std::integral_constant<int, 32>()); break;
+    case 64: f(std::integral_constant<int, 64>()); break;
+    case 128: f(std::integral_constant<int, 128>()); break;
+    case 256: f(std::integral_constant<int, 256>()); break;
+    case 512: f(std::integral_constant<int, 512>()); break;
+    default: f(std::integral_constant<int, 1024>()); break;
+  }
+}
+
+template <typename T, int C, bool INV>
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 2 : 1)
+k_multi_col(const __grid_constant__ WfMultiGrid r, const __grid_constant__ WfMultiArgs a) {
+  WfBlk kb;
+  const int q = wf_multi_block(r, kb);
+  wf_rg_switch(a.g[q].n, [&](auto n) {
+    constexpr int N = decltype(n)::value;
+    auto width = [&](auto w) {
+      constexpr int TC = decltype(w)::value;
+      if (threadIdx.x >= WfRegCol<T, C, N, TC>::THREADS) return;
+      if constexpr (INV) wf_rg_lb_colinv_map<T, C, N, TC>(a.g[q], a.b[q], a.lb[q], kb.y, kb.x);
+      else wf_rg_lb_colfwd_map<T, C, N, TC>(a.g[q], a.b[q], a.lb[q], kb.y, kb.x);
+    };
+    constexpr int A = wf_rg_tc(N, C, 1), B = wf_rg_tc(N, C, 2);
+    if (a.g[q].TC == A) width(std::integral_constant<int, A>());
+    else width(std::integral_constant<int, B>());
+  });
+}
+template <typename T>
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 2 : 1)
+k_multi_row(const __grid_constant__ WfMultiGrid r, const __grid_constant__ WfMultiArgs a) {
+  WfBlk kb;
+  const int q = wf_multi_block(r, kb);
+  if ((int)threadIdx.x >= 32 * (a.g[q].RB / wf_rg_rows(a.g[q].nx))) return;
+  wf_rg_switch(a.g[q].nx, [&](auto n) { wf_rg_lb_row_map<T, decltype(n)::value>(a.g[q], a.b[q], a.lb[q], kb.y, kb.x); });
+}
+
+// Shared memory of a problem's stages.
+template <typename T> inline size_t wf_multi_col_smem(const WfGeo& g) {
+  size_t sm = 0;
+  wfimpl::rg_length(g.n, [&](auto n) {
+    const bool wide = g.TC == wf_rg_tc(n(), g.C, 1);
+    if (g.C == 1) sm = wide ? WfRegCol<T, 1, n(), wf_rg_tc(n(), 1, 1)>::SMEM : WfRegCol<T, 1, n(), wf_rg_tc(n(), 1, 2)>::SMEM;
+    else sm = wide ? WfRegCol<T, 2, n(), wf_rg_tc(n(), 2, 1)>::SMEM : WfRegCol<T, 2, n(), wf_rg_tc(n(), 2, 2)>::SMEM;
+    return cudaSuccess;
+  });
+  return sm;
+}
+template <typename T> inline size_t wf_multi_row_smem(const WfGeo& g) {
+  size_t sm = 0;
+  wfimpl::rg_length(g.nx, [&](auto n) {
+    sm = WfRegRow<T, n()>::smem(g.RB / wf_rg_rows(g.nx));
+    return cudaSuccess;
+  });
+  return sm;
+}
+
+template <typename T, int C>
+cudaError_t wf_launch_multi_fft(const WfMultiArgs& a, int stage, cudaStream_t st) {
+  static int done[3] = {0, 0, 0};
+  const bool row = stage == 1;
+  const WfMultiGrid r = wf_multi_grid(a, [&](const WfGeo& g) { return row ? g.nrb : g.ntile; });
+  size_t sm = 0;
+  for (int q = 0; q < a.np; ++q) {
+    const size_t s = row ? wf_multi_row_smem<T>(a.g[q]) : wf_multi_col_smem<T>(a.g[q]);
+    if (s > sm) sm = s;
+  }
+  auto k = row ? k_multi_row<T> : stage == 0 ? k_multi_col<T, C, true> : k_multi_col<T, C, false>;
+  cudaError_t e = wfimpl::ensure_smem(k, WfRegCol<T, 1, 1024, wf_rg_tc(1024, 1, 1)>::SMEM, &done[stage]);  // the largest
+  if (e != cudaSuccess) return e;
+  k<<<r.start[a.np], 256, sm, st>>>(r, a);
+  return cudaGetLastError();
+}

@@ -158,9 +158,9 @@ __device__ __forceinline__ void wf_rg_pass2(V2<T>* v) {
 // Pass-1 twiddles of a length-N transform with radices R1, R2 into shared
 // memory: tw[q R2 + j] = exp(-2 pi i q j / N), from the table of WF_NT-th roots.
 template <typename T, int N, int R2>
-__device__ __forceinline__ void wf_rg_stage_tw(V2<T>* s_tw, const void* tw_) {
+__device__ __forceinline__ void wf_rg_stage_tw(V2<T>* s_tw, const void* tw_, int threads) {
   const V2<T>* roots = (const V2<T>*)tw_;
-  for (int i = threadIdx.x; i < N; i += blockDim.x) {
+  for (int i = threadIdx.x; i < N; i += threads) {
     const int q = i / R2, j = i - q * R2;
     s_tw[i] = roots[(q * j) * (WF_NT / N)];
   }
@@ -316,7 +316,7 @@ __device__ __forceinline__ void wf_rg_colinv(const WfGeo& geo, const V2<T>* src,
   const unsigned o0 = (unsigned)(c * N + g) * pitch + (unsigned)kx, step = K::G * pitch;
 #pragma unroll
   for (int m = 0; m < K::NV; ++m) v[m] = __ldcg(src + WF_CHK(o0 + m * step, C * N * pitch));
-  wf_rg_stage_tw<T, N, K::R2>(s_tw, tw_);
+  wf_rg_stage_tw<T, N, K::R2>(s_tw, tw_, K::THREADS);
   if (kx0 == 0 && col0) {
 #pragma unroll
     for (int m = 0; m < K::NV; ++m) {
@@ -351,7 +351,7 @@ __device__ __forceinline__ void wf_rg_colsim(const WfGeo& geo, const T* sp, V2<T
   const unsigned d0 = (unsigned)(c * N + g) * h + (unsigned)kx, dstep = K::G * h;
 #pragma unroll
   for (int m = 0; m < K::NV; ++m) v[m] = __ldcg(scr + WF_CHK(d0 + m * dstep, C * N * h));
-  wf_rg_stage_tw<T, N, K::R2>(s_tw, tw_);
+  wf_rg_stage_tw<T, N, K::R2>(s_tw, tw_, K::THREADS);
   wf_rg_cols<T, C, N, TC, -1>(v, xch + t, s_tw, g);
   wf_rg_pass2<T, N, K::R1, K::R2, K::NV, -1>(v);
   const T unit = (T)(1.0 / sqrt((double)N * (double)geo.nx));
@@ -382,7 +382,7 @@ __device__ __forceinline__ void wf_rg_colfwd_front(V2<T>* v, const WfGeo& geo, c
   const unsigned d0 = (unsigned)(c * N + g) * h + (unsigned)kx, dstep = K::G * h;
 #pragma unroll
   for (int m = 0; m < K::NV; ++m) v[m] = __ldcg(scr + WF_CHK(d0 + m * dstep, C * N * h));
-  wf_rg_stage_tw<T, N, K::R2>(s_tw, tw_);
+  wf_rg_stage_tw<T, N, K::R2>(s_tw, tw_, K::THREADS);
   wf_rg_cols<T, C, N, TC, -1>(v, xch + t, s_tw, g);
   const unsigned a0 = (unsigned)(c * N + g) * pitch + (unsigned)kx, astep = K::G * pitch;
   auto fetch = [&]() {
@@ -409,9 +409,9 @@ __device__ __forceinline__ V2<T> wf_rg_aux(int t, int g, int m) {
   return ((V2<T>*)wf_smem)[t + wf_rg_place<N, K::R2, K::NV, K::PITCH, K::S>(g, m)];
 }
 
-// Sum over the block of one double per thread (any number of whole warps);
-// valid in thread 0.
-__device__ __forceinline__ double wf_rg_block_sum(double v) {
+// Sum over the block's first `warps` warps (the others have left) of one double
+// per thread; valid in thread 0.
+__device__ __forceinline__ double wf_rg_block_sum(double v, int warps) {
   __shared__ double red[32];
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
@@ -420,7 +420,7 @@ __device__ __forceinline__ double wf_rg_block_sum(double v) {
   __syncthreads();
   double r = 0.0;
   if (threadIdx.x == 0)
-    for (int i = 0; i < (int)(blockDim.x >> 5); ++i) r += red[i];
+    for (int i = 0; i < warps; ++i) r += red[i];
   return r;
 }
 
@@ -477,9 +477,9 @@ __device__ __forceinline__ void wf_rg_colfwd(const WfGeo& geo, const V2<T>* src,
       }
     }
   }
-  const double s1 = wf_rg_block_sum(prior);
+  const double s1 = wf_rg_block_sum(prior, K::THREADS / 32);
   if (threadIdx.x == 0) part_b[(size_t)WF_SLOT_PRIOR * geo.maxblk + bx] = s1;
-  const double s2 = wf_rg_block_sum(out2);
+  const double s2 = wf_rg_block_sum(out2, K::THREADS / 32);
   if (threadIdx.x == 0) part_b[(size_t)WF_SLOT_OUT2 * geo.maxblk + bx] = s2;
 }
 
@@ -580,10 +580,16 @@ __device__ __forceinline__ void wf_rg_row_fft(V2<T>* v, V2<T>* xch, const V2<T>*
   }
 }
 
-// MODE as k_row.  Row block rb of map b; d, w, aux, out: whole arrays.
+//   MODE DATA / NODATA: c2r, r = d - x (or -x), wr = w r, data partial sum
+//     r.wr, r2c of wr, store packed rows back to scratch.
+//   MODE SIGNAL: c2r, write x to out (pixel layout).
+//   MODE SIM: c2r, out = (w > 0) ? x + aux : 0 (aux = noise).
+//   MODE RFFT: r2c of the pixel rows of aux (a white field), store to scratch.
+// Row block rb of map b, on the block's first `warps` warps; d, w, aux, out: whole
+// arrays.
 template <typename T, int MODE, int NX>
 __device__ __forceinline__ void wf_rg_row(const WfGeo& geo, V2<T>* scratch, const T* d, const T* w, const T* aux,
-                                          T* out, double* part, const void* tw_, int b, int rb) {
+                                          T* out, double* part, const void* tw_, int b, int rb, int warps) {
   typedef WfRegRow<T, NX> K;
   constexpr int h = NX / 2, NV = K::NV, G = K::G;
   extern __shared__ __align__(16) unsigned char wf_smem[];
@@ -591,7 +597,7 @@ __device__ __forceinline__ void wf_rg_row(const WfGeo& geo, V2<T>* scratch, cons
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, g = lane & (G - 1), t = lane / G;
   V2<T>* xch = s_tw + K::NTW + (wid * K::SEQ + t) * K::XCH;
   const int rows = geo.C * geo.n;
-  const int rt = 2 * ((rb * (int)(blockDim.x >> 5) + wid) * K::SEQ + t);
+  const int rt = 2 * ((rb * warps + wid) * K::SEQ + t), nth = 32 * warps;
   const bool ok = rt < rows;     // a sequence beyond the map computes on the first rows and stores nothing
   const int r0 = ok ? rt : 0;    // this sequence's rows r0, r0 + 1
   V2<T>* sc = scratch + ((size_t)b * rows + r0) * h;
@@ -633,13 +639,13 @@ __device__ __forceinline__ void wf_rg_row(const WfGeo& geo, V2<T>* scratch, cons
   {
     const V2<T>* roots = (const V2<T>*)tw_;
     if constexpr (MODE != WF_ROW_RFFT) {
-      for (int i = threadIdx.x; i < NX; i += blockDim.x) s_tw[i] = roots[((i / K::RB) * (i % K::RB)) * (WF_NT / NX)];
+      for (int i = threadIdx.x; i < NX; i += nth) s_tw[i] = roots[((i / K::RB) * (i % K::RB)) * (WF_NT / NX)];
     }
     if constexpr (K::RA != K::RB && (MODE == WF_ROW_RFFT || MODE == WF_ROW_DATA || MODE == WF_ROW_NODATA)) {
-      for (int i = threadIdx.x; i < NX; i += blockDim.x)
+      for (int i = threadIdx.x; i < NX; i += nth)
         s_tw[NX + i] = roots[((i / K::RA) * (i % K::RA)) * (WF_NT / NX)];
     } else if constexpr (MODE == WF_ROW_RFFT) {
-      for (int i = threadIdx.x; i < NX; i += blockDim.x) s_tw[i] = roots[((i / K::RA) * (i % K::RA)) * (WF_NT / NX)];
+      for (int i = threadIdx.x; i < NX; i += nth) s_tw[i] = roots[((i / K::RA) * (i % K::RA)) * (WF_NT / NX)];
     }
   }
   if constexpr (MODE == WF_ROW_DATA || MODE == WF_ROW_NODATA || MODE == WF_ROW_SIM) {
@@ -749,7 +755,39 @@ __device__ __forceinline__ void wf_rg_row(const WfGeo& geo, V2<T>* scratch, cons
     }
   }
   if constexpr (MODE == WF_ROW_DATA || MODE == WF_ROW_NODATA) {
-    const double s = wf_rg_block_sum(acc);
+    const double s = wf_rg_block_sum(acc, warps);
     if (threadIdx.x == 0) part[((size_t)b * WF_NSLOT + WF_SLOT_DATA) * geo.maxblk + rb] = s;
   }
+}
+
+// ---------------------------------------------------------------------------
+// The stages of the L-BFGS iteration on the direction P[next] of map bm, for a
+// block at column tile (row block) bx of its problem's own grid.
+// ---------------------------------------------------------------------------
+template <typename T, int C, int N, int TC>
+__device__ __forceinline__ void wf_rg_lb_colinv_map(const WfGeo& g, const WfBufs& b, const WfLbBufs& lb, int bm, int bx) {
+  const WfLbMap* M = lb.st + bm;
+  if (!M->active) return;
+  const size_t vsz = (size_t)C * N * g.h;
+  wf_rg_colinv<T, C, WF_IN_PK, N, TC>(g, (const V2<T>*)lb.ring + ((size_t)M->next * b.B + bm) * vsz,
+                                      (const T*)b.sp + (size_t)bm * b.sp_stride, (V2<T>*)b.scratch + (size_t)bm * vsz,
+                                      b.tw, bx * TC);
+}
+template <typename T, int NX>
+__device__ __forceinline__ void wf_rg_lb_row_map(const WfGeo& g, const WfBufs& b, const WfLbBufs& lb, int bm, int bx) {
+  if (!lb.st[bm].active) return;
+  wf_rg_row<T, WF_ROW_NODATA, NX>(g, (V2<T>*)b.scratch, nullptr, (const T*)b.w, nullptr, nullptr, b.part, b.tw, bm, bx,
+                                  g.RB / wf_rg_rows(NX));
+}
+template <typename T, int C, int N, int TC>
+__device__ __forceinline__ void wf_rg_lb_colfwd_map(const WfGeo& g, const WfBufs& b, const WfLbBufs& lb, int bm, int bx) {
+  const WfLbMap* M = lb.st + bm;
+  if (!M->active) return;
+  const size_t vsz = (size_t)C * N * g.h;
+  const int nx = M->next;
+  V2<T>* ring = (V2<T>*)lb.ring;
+  wf_rg_lb_colfwd<T, C, N, TC>(g, ring + ((size_t)nx * b.B + bm) * vsz, (const V2<T>*)lb.g + (size_t)bm * vsz,
+                               ring + ((size_t)(lb.m + nx) * b.B + bm) * vsz, (const T*)b.sp + (size_t)bm * b.sp_stride,
+                               (const V2<T>*)b.scratch + (size_t)bm * vsz,
+                               b.part + (size_t)bm * WF_NSLOT * g.maxblk, b.tw, bx * TC, bx);
 }

@@ -35,42 +35,25 @@ __global__ void __launch_bounds__(256, wf_rg_minb<T, WfReg<NX>::NV>(256))
 k_rg_row(WfGeo g, void* scratch_, const void* d_, const void* w_, const void* aux_, void* out_, double* part,
          const void* tw_) {
   wf_rg_row<T, MODE, NX>(g, (V2<T>*)scratch_, (const T*)d_, (const T*)w_, (const T*)aux_, (T*)out_, part, tw_,
-                         blockIdx.y, blockIdx.x);
+                         blockIdx.y, blockIdx.x, blockDim.x >> 5);
 }
 
-// The same stages on the direction P[next] of every map still iterating.
+// The same stages on the direction P[next] of every map still iterating (device
+// functions in wf_reg.cuh, shared with the launches over several problems).
 template <typename T, int C, int N, int TC>
 __global__ void __launch_bounds__(WfRegCol<T, C, N, TC>::THREADS, wf_rg_minb<T, WfReg<N>::NV>(WfRegCol<T, C, N, TC>::THREADS))
-k_rg_lb_colinv(WfGeo g, const T* sp_, long long sp_stride, void* scratch_, const void* tw_, WfLbBufs lb) {
-  const int b = blockIdx.y;
-  const WfLbMap* M = lb.st + b;
-  if (!M->active) return;
-  const size_t vsz = (size_t)C * N * g.h;
-  wf_rg_colinv<T, C, WF_IN_PK, N, TC>(g, (const V2<T>*)lb.ring + ((size_t)M->next * gridDim.y + b) * vsz,
-                                      sp_ + (size_t)b * sp_stride, (V2<T>*)scratch_ + (size_t)b * vsz, tw_,
-                                      blockIdx.x * TC);
+k_rg_lb_colinv(WfGeo g, WfBufs b, WfLbBufs lb) {
+  wf_rg_lb_colinv_map<T, C, N, TC>(g, b, lb, blockIdx.y, blockIdx.x);
 }
 template <typename T, int NX>
 __global__ void __launch_bounds__(256, wf_rg_minb<T, WfReg<NX>::NV>(256))
-k_rg_lb_row(WfGeo g, void* scratch_, const void* w_, double* part, const void* tw_, const WfLbMap* st) {
-  if (!st[blockIdx.y].active) return;
-  wf_rg_row<T, WF_ROW_NODATA, NX>(g, (V2<T>*)scratch_, nullptr, (const T*)w_, nullptr, nullptr, part, tw_, blockIdx.y,
-                                  blockIdx.x);
+k_rg_lb_row(WfGeo g, WfBufs b, WfLbBufs lb) {
+  wf_rg_lb_row_map<T, NX>(g, b, lb, blockIdx.y, blockIdx.x);
 }
 template <typename T, int C, int N, int TC>
 __global__ void __launch_bounds__(WfRegCol<T, C, N, TC>::THREADS, wf_rg_minb<T, WfReg<N>::NV>(WfRegCol<T, C, N, TC>::THREADS))
-k_rg_lb_colfwd(WfGeo g, const T* sp_, long long sp_stride, const void* scratch_, const void* tw_, WfLbBufs lb,
-               double* part) {
-  const int b = blockIdx.y;
-  const WfLbMap* M = lb.st + b;
-  if (!M->active) return;
-  const size_t vsz = (size_t)C * N * g.h;
-  const int nx = M->next;
-  const V2<T>* ring = (const V2<T>*)lb.ring;
-  wf_rg_lb_colfwd<T, C, N, TC>(g, ring + ((size_t)nx * gridDim.y + b) * vsz, (const V2<T>*)lb.g + (size_t)b * vsz,
-                               (V2<T>*)lb.ring + ((size_t)(lb.m + nx) * gridDim.y + b) * vsz,
-                               sp_ + (size_t)b * sp_stride, (const V2<T>*)scratch_ + (size_t)b * vsz,
-                               part + (size_t)b * WF_NSLOT * g.maxblk, tw_, blockIdx.x * TC, blockIdx.x);
+k_rg_lb_colfwd(WfGeo g, WfBufs b, WfLbBufs lb) {
+  wf_rg_lb_colfwd_map<T, C, N, TC>(g, b, lb, blockIdx.y, blockIdx.x);
 }
 
 namespace {
@@ -131,7 +114,7 @@ cudaError_t rg_lb_colinv_k(const WfGeo& g, const WfBufs& b, const WfLbBufs& lb, 
   auto k = k_rg_lb_colinv<T, C, N, TC>;
   cudaError_t e = rg_smem(k, K::SMEM, &done);
   if (e != cudaSuccess) return e;
-  k<<<dim3(g.ntile, b.B), K::THREADS, K::SMEM, st>>>(g, (const T*)b.sp, b.sp_stride, b.scratch, b.tw, lb);
+  k<<<dim3(g.ntile, b.B), K::THREADS, K::SMEM, st>>>(g, b, lb);
   return cudaGetLastError();
 }
 template <typename T, int C, int N, int TC>
@@ -141,7 +124,7 @@ cudaError_t rg_lb_colfwd_k(const WfGeo& g, const WfBufs& b, const WfLbBufs& lb, 
   auto k = k_rg_lb_colfwd<T, C, N, TC>;
   cudaError_t e = rg_smem(k, K::SMEM, &done);
   if (e != cudaSuccess) return e;
-  k<<<dim3(g.ntile, b.B), K::THREADS, K::SMEM, st>>>(g, (const T*)b.sp, b.sp_stride, b.scratch, b.tw, lb, b.part);
+  k<<<dim3(g.ntile, b.B), K::THREADS, K::SMEM, st>>>(g, b, lb);
   return cudaGetLastError();
 }
 template <typename T, int MODE, int NX>
@@ -203,7 +186,7 @@ cudaError_t wf_reg_lb_row(const WfGeo& g, const WfBufs& b, const WfLbBufs& lb, c
   cudaError_t e = rg_smem(k, K::smem(8), &done);
   if (e != cudaSuccess) return e;
   const int warps = g.RB / wf_rg_rows(NX);
-  k<<<dim3(g.nrb, b.B), 32 * warps, K::smem(warps), st>>>(g, b.scratch, b.w, b.part, b.tw, lb.st);
+  k<<<dim3(g.nrb, b.B), 32 * warps, K::smem(warps), st>>>(g, b, lb);
   return cudaGetLastError();
 }
 

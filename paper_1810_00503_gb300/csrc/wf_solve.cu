@@ -761,6 +761,7 @@ static wf_status choose_variant(wf_problem* p, WfSolver* S, cudaStream_t st) {
       if (shared && ck != base.colinv_kind) continue;
       int last_tc = -1;
       for (int di : divs) {
+        if (shared && di > 2) continue;  // the shared launches have two widths
         const WfGeo g = wf_geo_variant(base, ck, base.row_kind, di, 1, cp, 0);
         if (g.TC == last_tc) continue;  // no narrower tile possible
         last_tc = g.TC;
@@ -1333,18 +1334,34 @@ static cudaError_t any_refresh(wf_problem* p, cudaStream_t st) {
                                  : refresh<float>(p, wf_bufs(p), lb_bufs<float>(S), S->A, 0, S, st);
 }
 
-// One L-BFGS iteration of several problems: the streaming kernels, the active
-// counters' reset and the scalar step in launches shared by all (see
-// WfMultiArgs), the FFT stages per problem.
+// One L-BFGS iteration of several problems in shared launches (see
+// WfMultiArgs): the five kernels of iteration() plus the active counters'
+// reset and the scalar step, seven launches whatever the number of problems.  A
+// problem whose column stage alone has WF_MULTI_SOLO blocks runs its FFT stages in
+// launches of its own: they fill the chip, and are not held to the registers and
+// shared memory of the other lengths (64^2 to 1024^2, 48 maps each: 14.2 against
+// 15.4 ms for eight iterations; with a few small maps a launch of its own per
+// problem costs more, 3.5 us a node of the batch's graph, than it gains).
+#define WF_MULTI_SOLO 1024
 static_assert(WF_SW == 1, "the shared scalar launch takes one block per map");
 template <typename T>
 static cudaError_t multi_iteration(const WfMultiArgs& a, const WfMultiScalar& ms, cudaStream_t st) {
   cudaError_t e = wf_launch_multi_comb<T>(a, WF_LB1_FULL, st);
+  WfMultiArgs f;  // the problems whose FFT stages share launches
+  f.np = 0;
   for (int q = 0; q < a.np && e == cudaSuccess; ++q) {
+    if ((long long)a.g[q].ntile * a.b[q].B < WF_MULTI_SOLO) {
+      f.g[f.np] = a.g[q];
+      f.b[f.np] = a.b[q];
+      f.lb[f.np++] = a.lb[q];
+      continue;
+    }
     e = wf_launch_lb_colinv<T>(a.g[q], a.b[q], a.lb[q], st);
     if (e == cudaSuccess) e = wf_launch_lb_row<T>(a.g[q], a.b[q], a.lb[q], st);
     if (e == cudaSuccess) e = wf_launch_lb_colfwd<T>(a.g[q], a.b[q], a.lb[q], st);
   }
+  for (int stage = 0; stage < 3 && e == cudaSuccess && f.np > 0; ++stage)
+    e = f.g[0].C == 1 ? wf_launch_multi_fft<T, 1>(f, stage, st) : wf_launch_multi_fft<T, 2>(f, stage, st);
   if (e == cudaSuccess) e = wf_launch_multi_qdots<T>(a, st);
   if (e == cudaSuccess) {
     k_multi_zero<<<1, 32, 0, st>>>(ms);
@@ -1360,9 +1377,9 @@ static cudaError_t multi_iteration(const WfMultiArgs& a, const WfMultiScalar& ms
 // Several problems (typically one per map shape of a heterogeneous batch)
 // solved as one batch.  Every problem is started on its own stream (first
 // gradient).  When the problems share the working type and C (and no FFT-stage
-// variant is forced), an iteration of the whole batch shares its streaming and
-// scalar launches (multi_iteration), every problem on the register-resident
-// stages of WF_MULTI_VARIANT with its own tuned tile widths; otherwise each problem is
+// variant is forced), each iteration of the whole batch is seven shared
+// launches (multi_iteration), every problem on the register-resident stages of
+// WF_MULTI_VARIANT with its own tuned tile widths; otherwise each problem is
 // tuned freely and runs its own kernels, as a parallel branch per problem.  check_every iterations are
 // captured in one CUDA graph, so that each round is one graph launch for the
 // whole batch; the maps of every shape advance together and a problem whose

@@ -19,46 +19,6 @@
 
 #include "wf_api_internal.h"
 
-// Theta_fid,l: full-plane mean of P over band l (half-plane multiplicity 1 on
-// the kx = 0 and kx = nx/2 columns, 2 elsewhere; P is [C][ny][nx/2+1]).  One block; per-warp bins
-// ([warps][2 nb]: sums, then counts) summed in a fixed order, so the result is
-// the same on every run.
-template <typename S>
-__global__ void k_theta_fid(const S* P, const int16_t* band, int ny, int nx, int C, int nb, double* theta) {
-  extern __shared__ double sh[];
-  const int nw = blockDim.x >> 5, w = threadIdx.x >> 5;
-  for (int i = threadIdx.x; i < 2 * nb * nw; i += blockDim.x) sh[i] = 0.0;
-  __syncthreads();
-  const int h = nx / 2;
-  const size_t tot = (size_t)C * ny * (h + 1);
-  double* bins = sh + (size_t)w * 2 * nb;
-  for (size_t i0 = 0; i0 < tot; i0 += blockDim.x) {  // uniform trip count across the block
-    const size_t i = i0 + threadIdx.x;
-    int l = -1;
-    double wt = 0.0, pv = 0.0;
-    if (i < tot) {
-      l = band[i];
-      if (l >= nb) l = -1;
-      if (l >= 0) {
-        const int kx = (int)(i % (h + 1));
-        wt = (kx == 0 || kx == h) ? 1.0 : 2.0;
-        pv = wt * (double)P[i];
-      }
-    }
-    wf_warp_bin_add(bins, l, pv);
-    wf_warp_bin_add(bins + nb, l, wt);
-  }
-  __syncthreads();
-  for (int l = threadIdx.x; l < nb; l += blockDim.x) {
-    double sum = 0.0, cnt = 0.0;
-    for (int q = 0; q < nw; ++q) {
-      sum += sh[(size_t)q * 2 * nb + l];
-      cnt += sh[(size_t)q * 2 * nb + nb + l];
-    }
-    theta[l] = cnt > 0.0 ? sum / cnt : 0.0;
-  }
-}
-
 // P restricted to each band: out[l][i] = band[i] == l ? P[i] : 0; with lo > 0
 // one more table, P on the bands lo and above (the B bands of the
 // leakage-bias form): out[nb][i] = band[i] >= lo ? P[i] : 0.
@@ -365,14 +325,12 @@ extern "C" wf_status bandpower_estimate_rect(wf_handle* h, const wf_map* data, i
   const int nF = nR * nfd, Btot = 1 + J + nF;
   Scope sc(h);
   // Theta_fid and the band-restricted power tables
-  double* theta = nullptr;
-  BP_OK(wf_alloc(h, (void**)&theta, sizeof(double) * nb, "theta_fid"));
+  double* theta = nullptr;  // then the work space of its sums
+  const WfGeo geo = wf_make_geo(ny, nx, C, 1);
+  BP_OK(wf_alloc(h, (void**)&theta, sizeof(double) * nb * (1 + 2 * (size_t)wf_band_nblk(geo)), "theta_fid"));
   sc.add(theta);
-  if (dtype == WF_F64)
-    k_theta_fid<double><<<1, 1024, 64 * nb * sizeof(double), st>>>((const double*)data->P, in->band, ny, nx, C, nb, theta);
-  else
-    k_theta_fid<float><<<1, 1024, 64 * nb * sizeof(double), st>>>((const float*)data->P, in->band, ny, nx, C, nb, theta);
-  BP_TRY(cudaGetLastError());
+  if (dtype == WF_F64) BP_TRY(wf_launch_theta_fid<double>(geo, data->P, in->band, nb, theta + nb, theta, st));
+  else BP_TRY(wf_launch_theta_fid<float>(geo, data->P, in->band, nb, theta + nb, theta, st));
   void* Pl = nullptr;
   BP_OK(wf_alloc(h, &Pl, nsp * (nb + (L > 0)) * delt, "band-restricted power"));
   sc.add(Pl);

@@ -301,6 +301,11 @@ cudaError_t wf_launch_simulate(const WfGeo& g, const WfBufs& b, const void* z, c
 template <typename T>
 cudaError_t wf_launch_band_energy(const WfGeo& g, int B, const void* s, const int16_t* band,
                                   const double* theta, int n_bands, double* bpart, double* E, cudaStream_t st);
+// Theta_fid,l: full-plane mean of P ([C][ny][nx/2+1], type S) over band l (nb <=
+// 64); work: 2 * wf_band_nblk(g) * nb doubles.
+template <typename S>
+cudaError_t wf_launch_theta_fid(const WfGeo& g, const void* P, const int16_t* band, int nb, double* work,
+                                double* theta, cudaStream_t st);
 // L-BFGS kernels.  Streaming-kernel modes: full iteration, materialise only, dots only.
 enum { WF_LB1_FULL = 0, WF_LB1_MATERIALIZE = 1, WF_LB1_DOTS = 2 };
 // The steps taken but not yet added to s are folded in one pass once this

@@ -46,12 +46,33 @@ template <class F> inline cudaError_t rg_length(int n, F&& f) {
   return cudaErrorInvalidValue;
 }
 
-// Deterministic band sums of standard-layout spectra (k_band_reduce, then
-// k_band_final); bpart holds B * wf_band_nblk(g) * nb doubles.
+// Launch of k_band_priv over nblk blocks of each of B maps.
+template <typename T, int MODE>
+cudaError_t band_priv(int rows, int hp, int nblk, int B, const void* s, const void* grad, const int16_t* band, int nb,
+                      double* part, cudaStream_t st) {
+  static int done = 0;
+  auto k = k_band_priv<T, MODE>;
+  cudaError_t e = ensure_smem(k, sizeof(double) * WF_BAND_THREADS * WF_BAND_PRIV, &done);
+  if (e != cudaSuccess) return e;
+  int tx = 1;
+  while (tx < hp && tx < WF_BAND_THREADS) tx *= 2;
+  k<<<dim3(nblk, B), WF_BAND_THREADS, sizeof(double) * WF_BAND_THREADS * nb, st>>>(rows, hp, tx, s, (const V2<T>*)grad,
+                                                                                   band, nb, part);
+  return cudaGetLastError();
+}
+
+// Deterministic band sums of standard-layout spectra (k_band_priv or
+// k_band_reduce, then k_band_final); bpart holds B * wf_band_nblk(g) * nb doubles.
 template <typename T, int MODE>
 cudaError_t band_sums(const WfGeo& g, int B, const void* s, const void* grad, const int16_t* band, int nb,
                       const double* theta, double* bpart, double* out, cudaStream_t st) {
   const int nblk = wf_band_nblk(g);
+  if (nb <= WF_BAND_PRIV) {
+    cudaError_t e = band_priv<T, MODE>(g.C * g.n, g.h + 1, nblk, B, s, grad, band, nb, bpart, st);
+    if (e != cudaSuccess) return e;
+    k_band_final<<<B, 128, 0, st>>>(bpart, nblk, nb, theta, out);
+    return cudaGetLastError();
+  }
   const size_t sm = sizeof(double) * (WF_THREADS / 32) * (size_t)nb;
   if (sm > 48 * 1024) {
     cudaError_t e = cudaFuncSetAttribute(k_band_reduce<T, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
@@ -242,6 +263,17 @@ inline int grid1d(size_t total, int cap) {
                                        cudaStream_t st) {
     return wfimpl::band_sums<T, 0>(g, B, s, nullptr, band, n_bands, theta, bpart, E, st);
   }
+  template <typename S>
+  cudaError_t wf_launch_theta_fid(const WfGeo& g, const void* P, const int16_t* band, int nb, double* work,
+                                  double* theta, cudaStream_t st) {
+    const int nblk = wf_band_nblk(g), rows = g.C * g.n;
+    double* cnt = work + (size_t)nblk * nb;
+    cudaError_t e = wfimpl::band_priv<S, 2>(rows, g.h + 1, nblk, 1, P, nullptr, band, nb, work, st);
+    if (e == cudaSuccess) e = wfimpl::band_priv<S, 3>(rows, g.h + 1, nblk, 1, P, nullptr, band, nb, cnt, st);
+    if (e != cudaSuccess) return e;
+    k_theta_final<<<1, 64, 0, st>>>(work, cnt, nblk, nb, theta);
+    return cudaGetLastError();
+  }
   template <typename T>
   cudaError_t wf_launch_pack(const WfGeo& g, int B, const void* in, void* out,
                                 cudaStream_t st) {
@@ -339,6 +371,8 @@ cudaError_t wf_launch_eval_pk(const WfGeo& g, const WfBufs& b, const void* src, 
                                              const void*, void*, cudaStream_t);                    \
   template cudaError_t wf_launch_band_energy<T>(const WfGeo&, int, const void*, const int16_t*,    \
                                                 const double*, int, double*, double*, cudaStream_t); \
+  template cudaError_t wf_launch_theta_fid<T>(const WfGeo&, const void*, const int16_t*, int, double*, double*, \
+                                              cudaStream_t);                                         \
   template cudaError_t wf_launch_pack<T>(const WfGeo&, int, const void*, void*, cudaStream_t);     \
   template cudaError_t wf_launch_unpack<T>(const WfGeo&, int, const void*, void*, cudaStream_t);    \
   template cudaError_t wf_launch_eval_pk<T>(const WfGeo&, const WfBufs&, const void*, void*,       \

@@ -5,7 +5,7 @@
 //   k_lb_comb   s, g += a (P, Q) of the previous step; p = direction; <g, .>
 //   k_lb_colinv, k_lb_row, k_lb_colfwd   q = H p and <q,q>, <p,q>, <g,q>, <g,p>
 //   k_lb_qdots  <q, Q_i>
-//   k_lb_scalar (one warp per map) exact step a = -g.p / p.Hp along p (the
+//   k_lb_scalar (one block per map) exact step a = -g.p / p.Hp along p (the
 //             objective is quadratic, so this is the point a Wolfe line search
 //             converges to), chi^2 update, Gram-matrix update of the new pair
 //             (s, y) = (a p, a q), convergence test, and the two-loop recursion
@@ -83,7 +83,7 @@ enum { WF_RES_CHI2 = 0, WF_RES_GG, WF_RES_SS, WF_RES_CERT, WF_RES_ITERS, WF_RES_
 
 enum { WF_PH_ITER = 0, WF_PH_REFRESH = 1 };
 
-#define WF_SW 1                        // warps (maps) per block of the scalar kernel
+#define WF_ST 256                      // threads per map (block) of the scalar kernel
 #define WF_SCAL_SLOTS (6 + 3 * WF_MAXM)  // partial-sum slots one scalar step reads at most
 
 // Sum over the nb block partials of one slot (every lane gets the total).
@@ -96,69 +96,82 @@ __device__ __forceinline__ double wf_warp_slot(const double* pb, int slot, int n
   return v;
 }
 
-__device__ __forceinline__ double wf_warp_sum(double v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
+// Gram matrices of a map's stored vectors in shared memory (rows and columns < m).
+struct WfGram {
+  double PP[WF_MAXM][WF_MAXM + 1], PQ[WF_MAXM][WF_MAXM + 1], QQ[WF_MAXM][WF_MAXM + 1];
+};
 
 // Block partials of ns slots: out[k] = sum_i pb[slots[k] * maxblk + i], i < cnt[k].
-// Every lane first sums its stride-32 share of every slot (independent loads),
-// then lane k adds the 32 shares of slot k in lane order: a fixed order, so
-// the result is deterministic.
+// Warp w takes the slots w, w + warps, ..: every lane first sums its stride-32
+// share of a slot (independent loads, four sums), then thread k adds the 32 shares
+// of slot k in lane order: a fixed order, so the result is deterministic.  The
+// caller synchronises the block before out is read.
 __device__ void wf_gather_slots(const double* pb, int maxblk, const int* slots, const int* cnt, int ns,
                                 double (*red)[33], double* out) {
-  const int lane = threadIdx.x & 31;
-  for (int k = 0; k < ns; ++k) {
+  const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  for (int k = threadIdx.x >> 5; k < ns; k += nw) {
     const double* src = pb + (size_t)slots[k] * maxblk;
-    double v = 0.0;
-    for (int i = lane; i < cnt[k]; i += 32) v += src[i];
-    red[k][lane] = v;
+    const int n = cnt[k];
+    double v[4] = {0.0, 0.0, 0.0, 0.0};
+    for (int i = lane; i < n; i += 128) {
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (i + 32 * u < n) v[u] += src[i + 32 * u];
+    }
+    red[k][lane] = (v[0] + v[1]) + (v[2] + v[3]);
   }
-  __syncwarp();
-  for (int k = lane; k < ns; k += 32) {
+  __syncthreads();
+  for (int k = threadIdx.x; k < ns; k += blockDim.x) {
     double v = 0.0;
     for (int l = 0; l < 32; ++l) v += red[k][l];
     out[k] = v;
   }
-  __syncwarp();
 }
 
 // Two-loop recursion on coefficients (Nocedal & Wright, Alg. 7.4): r = H_k g
 // expressed over the basis {g, P_i, Q_i}; the direction is p = -r.  Lane l
-// holds the coefficients of history slot l (m <= 32); each step of the two
-// loops is one warp sum over the stored pairs.  Called by all 32 lanes.
-__device__ void wf_two_loop(WfLbMap& M, int m, int lane) {
+// holds the coefficients of history slot l (m <= 32) and the inner product its
+// own step will need, <P_l, r> in the first loop and <Q_l, r> in the second: a
+// step broadcasts one new coefficient and every lane adds its product with a
+// Gram column, so no step waits for a sum over the warp, and the reciprocals
+// rho_l are taken once, together (an FP64 instruction holds a warp's unit for 64
+// cycles: with a warp sum and a division a step, the loops took 20 us).
+// Called by all 32 lanes of one warp.
+__device__ void wf_two_loop(WfLbMap& M, const WfGram& G, int m, int lane) {
   const int np = M.npairs, head = M.head;
   const bool act = np > 0 && lane < m && (head - lane + m) % m < np;  // slot `lane` holds a stored pair
-  double cP = 0.0, cQ = 0.0, aa = 0.0, cg = 1.0;
-  for (int q = 0; q < np; ++q) {  // newest to oldest
+  const unsigned full = 0xffffffffu;
+  double cP = 0.0, cQ = 0.0, aa = 0.0, cg = 1.0, ra = 0.0, al = 0.0, d = 0.0;
+  if (act) {
+    al = M.alpha[lane];
+    ra = 1.0 / (al * al * G.PQ[lane][lane]) * al;
+    d = M.gP[lane];
+  }
+  for (int q = 0; q < np; ++q) {  // newest to oldest: d = <P_lane, r>
     const int i = (head - q + m) % m;
-    const double t = act ? cP * M.PP[i * WF_MAXM + lane] + cQ * M.PQ[i * WF_MAXM + lane] : 0.0;
-    const double d = cg * M.gP[i] + wf_warp_sum(t);
-    const double ai = M.alpha[i];
-    const double rho = 1.0 / (ai * ai * M.PQ[i * WF_MAXM + i]);
-    const double a = rho * ai * d;
     if (lane == i) {
-      aa = a;
-      cQ -= a * ai;
+      aa = ra * d;
+      cQ = -aa * al;
     }
+    const double c = __shfl_sync(full, cQ, i);
+    if (act) d += c * G.PQ[lane][i];
   }
   double gamma = 1.0;
-  if (np > 0) gamma = M.PQ[head * WF_MAXM + head] / M.QQ[head * WF_MAXM + head];
+  if (np > 0) gamma = G.PQ[head][head] / G.QQ[head][head];
   cg *= gamma;
-  cP *= gamma;
   cQ *= gamma;
+  double e = act ? cg * M.gQ[lane] : 0.0;  // <Q_lane, r>
+  for (int q = 0; q < np; ++q) {
+    const int i = (head - q + m) % m;
+    const double c = __shfl_sync(full, cQ, i);
+    if (act) e += c * G.QQ[lane][i];
+  }
   for (int q = np - 1; q >= 0; --q) {  // oldest to newest
     const int i = (head - q + m) % m;
-    const double t = act ? cP * M.PQ[lane * WF_MAXM + i] + cQ * M.QQ[i * WF_MAXM + lane] : 0.0;
-    const double d = cg * M.gQ[i] + wf_warp_sum(t);
-    const double ai = M.alpha[i];
-    const double rho = 1.0 / (ai * ai * M.PQ[i * WF_MAXM + i]);
-    const double beta = rho * ai * d;
-    if (lane == i) cP += ai * (aa - beta);
+    if (lane == i) cP = al * (aa - ra * e);
+    const double c = __shfl_sync(full, cP, i);
+    if (act) e += c * G.PQ[i][lane];
   }
-  __syncwarp();  // every lane has read the old coefficients' Gram entries
   if (lane == 0) {
     M.dg = -cg;
     M.next = (head + 1) % m;
@@ -214,39 +227,55 @@ __device__ double wf_wolfe_step(double d0, double c, double c1, double c2) {
   return a;
 }
 
-// One warp per map.  ITER: exact or Wolfe step along p, chi^2 and Gram-matrix
-// update of the new pair, convergence test, two-loop for the next direction.
-// REFRESH: true chi^2 and gradient dots after a full evaluation.
+// One block per map: all its warps add up the partial sums and bring the Gram
+// matrices to shared memory, the first one then does the step.  ITER: exact or
+// Wolfe step along p, chi^2 and Gram-matrix update of the new pair, convergence
+// test, two-loop for the next direction.  REFRESH: true chi^2 and gradient dots
+// after a full evaluation.
+// FP64 latency bounds it (see wf_two_loop): 22 us on a map of 512^2 with ten pairs
+// and 28 us on one of 1024^2, where one warp per map had taken 50 and 64 us.
 __device__ __forceinline__ void wf_lb_scalar(WfLbMap* st, const double* part, const WfScalarArgs& A, int b,
                                              int* nact) {
   __shared__ double red[WF_SCAL_SLOTS][33];
   __shared__ double S[WF_SCAL_SLOTS];
   __shared__ int slots[WF_SCAL_SLOTS], cnt[WF_SCAL_SLOTS];
-  const int lane = threadIdx.x & 31;
+  __shared__ WfGram G;
+  const int tid = threadIdx.x, lane = tid & 31;
   WfLbMap& M = st[b];
   const double* pb = part + (size_t)b * WF_NSLOT * A.maxblk;
   const int m = A.m;
+  const int active = M.active, status = M.status, np0 = M.npairs, head = M.head;
   // Steps the streaming pass just folded into s (the rule of k_lb_comb): all of
   // them before a refresh and for a map that had stopped, otherwise all once
   // wf_sfold(m) have gathered.
-  if (lane == 0 && (A.phase != WF_PH_ITER || !M.active || M.k - M.s_k >= wf_sfold(m))) M.s_k = M.k;
-  __syncwarp();
-  if (M.status == WF_ETIMEOUT) {  // a bounded device wait gave up on this map's data
-    if (lane == 0) {
+  const bool folded = A.phase != WF_PH_ITER || !active || M.k - M.s_k >= wf_sfold(m);
+  __syncthreads();  // every thread has read the state this block changes
+  if (tid == 0 && folded) M.s_k = M.k;
+  if (status == WF_ETIMEOUT) {  // a bounded device wait gave up on this map's data
+    if (tid == 0) {
       M.active = 0;
       M.pend_alpha = 0.0;
     }
     return;
   }
-  if (A.phase == WF_PH_ITER) {
-    if (!M.active) {
-      if (lane == 0) M.pend_alpha = 0.0;
-      return;
+  if (A.phase == WF_PH_ITER && !active) {
+    if (tid == 0) M.pend_alpha = 0.0;
+    return;
+  }
+  if (np0 > 0 && !(A.phase != WF_PH_ITER && A.init))
+    for (int k = tid; k < m * WF_MAXM; k += blockDim.x) {
+      const int i = k / WF_MAXM, l = k % WF_MAXM;
+      if (l < m) {
+        G.PP[i][l] = M.PP[k];
+        G.PQ[i][l] = M.PQ[k];
+        G.QQ[i][l] = M.QQ[k];
+      }
     }
-    const int np = M.npairs, head = M.head, nx = M.next;
+  if (A.phase == WF_PH_ITER) {
+    const int np = np0, nx = M.next;
     // slot list: 0 GG, 1 QQ, 2 PQ, 3 GQN, 4 GPN, 5 PP, then per stored pair q:
     // 6 + 3q GP, 7 + 3q GQ, 8 + 3q QQI (of slot (head - q) mod m)
-    if (lane == 0) {
+    if (tid == 0) {
       const int fixed[6] = {WF_SLOT_GG, WF_SLOT_QQ, WF_SLOT_PQ, WF_SLOT_GQN, WF_SLOT_GPN, WF_SLOT_PP};
       for (int k = 0; k < 6; ++k) {
         slots[k] = fixed[k];
@@ -260,8 +289,10 @@ __device__ __forceinline__ void wf_lb_scalar(WfLbMap* st, const double* part, co
         cnt[6 + 3 * q] = cnt[7 + 3 * q] = cnt[8 + 3 * q] = A.ncomb;
       }
     }
-    __syncwarp();
+    __syncthreads();
     wf_gather_slots(pb, A.maxblk, slots, cnt, 6 + 3 * np, red, S);
+    __syncthreads();
+    if (tid >= 32) return;
     const double ggk = S[0], qq = S[1], pq = S[2], gq = S[3], gp = S[4], pp = S[5];
     // position of slot `lane` among the stored pairs (newest first), if stored
     const int ql = (head - lane + m) % m;
@@ -292,8 +323,8 @@ __device__ __forceinline__ void wf_lb_scalar(WfLbMap* st, const double* part, co
       double a = M.dg * gPk, c = M.dg * gQk;
       for (int u = 0; u < np; ++u) {
         const int l = (head - u + m) % m;
-        a += M.dP[l] * M.PP[l * WF_MAXM + i] + M.dQ[l] * M.PQ[i * WF_MAXM + l];
-        c += M.dP[l] * M.PQ[l * WF_MAXM + i] + M.dQ[l] * M.QQ[l * WF_MAXM + i];
+        a += M.dP[l] * G.PP[l][i] + M.dQ[l] * G.PQ[i][l];
+        c += M.dP[l] * G.PQ[l][i] + M.dQ[l] * G.QQ[l][i];
       }
       rowPP = a;
       rowPQ = c;
@@ -301,11 +332,11 @@ __device__ __forceinline__ void wf_lb_scalar(WfLbMap* st, const double* part, co
     __syncwarp();  // all reads of the old Gram entries are done
     if (act && lane != nx) {
       const int i = lane;
-      M.PP[nx * WF_MAXM + i] = M.PP[i * WF_MAXM + nx] = rowPP;
-      M.PQ[nx * WF_MAXM + i] = rowPQ;  // <p, Q_i>
-      M.PQ[i * WF_MAXM + nx] = rowPQ;  // <P_i, H p> = <H P_i, p>
+      M.PP[nx * WF_MAXM + i] = M.PP[i * WF_MAXM + nx] = G.PP[nx][i] = G.PP[i][nx] = rowPP;
+      // <p, Q_i>, and <P_i, H p> = <H P_i, p>
+      M.PQ[nx * WF_MAXM + i] = M.PQ[i * WF_MAXM + nx] = G.PQ[nx][i] = G.PQ[i][nx] = rowPQ;
       const double qqi = S[8 + 3 * ql];
-      M.QQ[nx * WF_MAXM + i] = M.QQ[i * WF_MAXM + nx] = qqi;
+      M.QQ[nx * WF_MAXM + i] = M.QQ[i * WF_MAXM + nx] = G.QQ[nx][i] = G.QQ[i][nx] = qqi;
       // dot products of g_{k+1} = g_k + alpha q with the stored vectors
       M.gP[i] = gPk + alpha * rowPQ;
       M.gQ[i] = gQk + alpha * qqi;
@@ -315,9 +346,9 @@ __device__ __forceinline__ void wf_lb_scalar(WfLbMap* st, const double* part, co
       M.evals += 1;
       M.chi2_prev = M.chi2;
       M.chi2 = M.chi2 + alpha * gp + 0.5 * alpha * alpha * pq;
-      M.PP[nx * WF_MAXM + nx] = pp;
-      M.PQ[nx * WF_MAXM + nx] = pq;
-      M.QQ[nx * WF_MAXM + nx] = qq;
+      M.PP[nx * WF_MAXM + nx] = G.PP[nx][nx] = pp;
+      M.PQ[nx * WF_MAXM + nx] = G.PQ[nx][nx] = pq;
+      M.QQ[nx * WF_MAXM + nx] = G.QQ[nx][nx] = qq;
       M.gP[nx] = gp + alpha * pq;
       M.gQ[nx] = gq + alpha * qq;
       double gg = ggk + 2.0 * alpha * gq + alpha * alpha * qq;
@@ -347,14 +378,14 @@ __device__ __forceinline__ void wf_lb_scalar(WfLbMap* st, const double* part, co
     done = __shfl_sync(0xffffffffu, done, 0);
     __syncwarp();
     if (!done) {
-      wf_two_loop(M, m, lane);
+      wf_two_loop(M, G, m, lane);
       if (lane == 0) atomicAdd(nact, 1);
     }
     return;
   }
   // WF_PH_REFRESH: true chi^2 and gradient at the current state, exact dots.
-  const int np = A.init ? 0 : M.npairs, head = M.head;
-  if (lane == 0) {
+  const int np = A.init ? 0 : np0;
+  if (tid == 0) {
     slots[0] = WF_SLOT_PRIOR;
     cnt[0] = A.ntile;
     slots[1] = WF_SLOT_DATA;
@@ -368,8 +399,10 @@ __device__ __forceinline__ void wf_lb_scalar(WfLbMap* st, const double* part, co
       cnt[3 + 2 * q] = cnt[4 + 2 * q] = A.ncomb;
     }
   }
-  __syncwarp();
+  __syncthreads();
   wf_gather_slots(pb, A.maxblk, slots, cnt, 3 + 2 * np, red, S);
+  __syncthreads();
+  if (tid >= 32) return;
   const double prior = S[0], data = S[1], gg = S[2];
   bool go = false;
   if (lane == 0) {
@@ -406,18 +439,18 @@ __device__ __forceinline__ void wf_lb_scalar(WfLbMap* st, const double* part, co
   go = __shfl_sync(0xffffffffu, go, 0);
   __syncwarp();
   if (go) {
-    wf_two_loop(M, m, lane);
+    wf_two_loop(M, G, m, lane);
     if (lane == 0) atomicAdd(nact, 1);
   }
 }
 
-__global__ void __launch_bounds__(32 * WF_SW)
+__global__ void __launch_bounds__(WF_ST)
 k_lb_scalar(WfLbMap* st, const double* part, WfScalarArgs A, int B, int* nact) {
   if ((int)blockIdx.x < B) wf_lb_scalar(st, part, A, blockIdx.x, nact);
 }
 
 // The scalar step of several problems in one launch (wf_map_solve_many): one
-// block (warp) per map of every problem, problem q's maps at blocks
+// block per map of every problem, problem q's maps at blocks
 // start[q] .. start[q+1] - 1; and the zeroing of their active counters.
 struct WfMultiScalar {
   int np;
@@ -427,7 +460,7 @@ struct WfMultiScalar {
   int* nact[WF_MULTI_MAX];
   WfScalarArgs A[WF_MULTI_MAX];
 };
-__global__ void __launch_bounds__(32 * WF_SW) k_multi_scalar(const __grid_constant__ WfMultiScalar ms) {
+__global__ void __launch_bounds__(WF_ST) k_multi_scalar(const __grid_constant__ WfMultiScalar ms) {
   const int bid = blockIdx.x;
   int q = 0;
   while (q + 1 < ms.np && bid >= ms.start[q + 1]) ++q;
@@ -440,8 +473,7 @@ __global__ void k_multi_zero(const __grid_constant__ WfMultiScalar ms) {
 // Final statistics from the closing true evaluation: [k, evals, status, chi2, gnorm_rel].
 __global__ void k_lb_final(const WfLbMap* st, const double* part, int ntile, int nrb, int maxblk, int B,
                            double* out) {
-  const int w = threadIdx.x >> 5;
-  const int b = blockIdx.x * WF_SW + w;
+  const int b = blockIdx.x;
   if (b >= B) return;
   const double* pb = part + (size_t)b * WF_NSLOT * maxblk;
   const double prior = wf_warp_slot(pb, WF_SLOT_PRIOR, ntile, maxblk);
@@ -590,7 +622,7 @@ static cudaError_t iteration(const wf_problem* p, const WfBufs& b, const WfLbBuf
   if (e == cudaSuccess) e = wf_launch_lb_qdots<T>(p->g, b, lb, st);
   if (e == cudaSuccess) e = cudaMemsetAsync(S->nact, 0, sizeof(int), st);
   if (e == cudaSuccess) {
-    k_lb_scalar<<<(p->count + WF_SW - 1) / WF_SW, 32 * WF_SW, 0, st>>>(lb.st, b.part, A, p->count, S->nact);
+    k_lb_scalar<<<p->count, WF_ST, 0, st>>>(lb.st, b.part, A, p->count, S->nact);
     e = cudaGetLastError();
   }
   return e;
@@ -609,7 +641,7 @@ static cudaError_t refresh(const wf_problem* p, const WfBufs& b, const WfLbBufs&
     A.init = init;
     A.ntile = p->gp.ntile;
     A.nrb = p->gp.nrb;
-    k_lb_scalar<<<(p->count + WF_SW - 1) / WF_SW, 32 * WF_SW, 0, st>>>(lb.st, b.part, A, p->count, S->nact);
+    k_lb_scalar<<<p->count, WF_ST, 0, st>>>(lb.st, b.part, A, p->count, S->nact);
     e = cudaGetLastError();
   }
   return e;
@@ -930,7 +962,7 @@ static wf_status start_impl(wf_problem* p, const wf_opts* o, const void* s0, con
     WfScalarArgs Ai = A;
     Ai.phase = WF_PH_REFRESH;
     Ai.init = 1;
-    k_lb_scalar<<<(p->count + WF_SW - 1) / WF_SW, 32 * WF_SW, 0, st>>>(lb.st, b.part, Ai, p->count, S->nact);
+    k_lb_scalar<<<p->count, WF_ST, 0, st>>>(lb.st, b.part, Ai, p->count, S->nact);
     WF_TRY(cudaGetLastError());
   } else {
     WF_TRY(refresh<T>(p, b, lb, A, 1, S, st));
@@ -1006,7 +1038,7 @@ static wf_status finish_impl(wf_problem* p, void* s_out, void* x_out, wf_solve_s
   WfLbBufs lb = lb_bufs<T>(S);
   WF_TRY(wf_launch_lb_comb<T>(p->g, b, lb, WF_LB1_MATERIALIZE, st));
   WF_TRY(wf_launch_eval_pk<T>(p->gp, b, lb.s, lb.g, st));
-  k_lb_final<<<(p->count + WF_SW - 1) / WF_SW, 32 * WF_SW, 0, st>>>(lb.st, b.part, p->gp.ntile, p->gp.nrb,
+  k_lb_final<<<p->count, 32, 0, st>>>(lb.st, b.part, p->gp.ntile, p->gp.nrb,
                                                                     p->gp.maxblk, p->count, S->stats_dev);
   WF_TRY(cudaGetLastError());
   if (s_out) WF_TRY(wf_launch_unpack<T>(p->g, p->count, S->s, s_out, st));
@@ -1206,7 +1238,7 @@ static wf_status profile_impl(wf_problem* p, int n_iter, float* ms) {
     if (e == cudaSuccess) e = cudaEventRecord(ev[5], st);
     if (e == cudaSuccess) e = cudaMemsetAsync(S->nact, 0, sizeof(int), st);
     if (e == cudaSuccess) {
-      k_lb_scalar<<<(p->count + WF_SW - 1) / WF_SW, 32 * WF_SW, 0, st>>>(lb.st, b.part, S->A, p->count, S->nact);
+      k_lb_scalar<<<p->count, WF_ST, 0, st>>>(lb.st, b.part, S->A, p->count, S->nact);
       e = cudaGetLastError();
     }
     if (e == cudaSuccess) e = cudaEventRecord(ev[6], st);
@@ -1343,7 +1375,6 @@ static cudaError_t any_refresh(wf_problem* p, cudaStream_t st) {
 // 15.4 ms for eight iterations; with a few small maps a launch of its own per
 // problem costs more, 3.5 us a node of the batch's graph, than it gains).
 #define WF_MULTI_SOLO 1024
-static_assert(WF_SW == 1, "the shared scalar launch takes one block per map");
 template <typename T>
 static cudaError_t multi_iteration(const WfMultiArgs& a, const WfMultiScalar& ms, cudaStream_t st) {
   cudaError_t e = wf_launch_multi_comb<T>(a, WF_LB1_FULL, st);
@@ -1368,7 +1399,7 @@ static cudaError_t multi_iteration(const WfMultiArgs& a, const WfMultiScalar& ms
     e = cudaGetLastError();
   }
   if (e == cudaSuccess) {
-    k_multi_scalar<<<ms.start[ms.np], 32 * WF_SW, 0, st>>>(ms);
+    k_multi_scalar<<<ms.start[ms.np], WF_ST, 0, st>>>(ms);
     e = cudaGetLastError();
   }
   return e;

@@ -689,6 +689,10 @@ extern "C" wf_status wf_eval_any(wf_handle* h, int B, int C, int ny, int nx, int
   if (f64) any_tiles<double>(G);
   else any_tiles<float>(G);
   const size_t vsz = (size_t)C * ny * G.h1;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;  // the call synchronises: refuse before it allocates
+  cudaError_t ce = cudaStreamIsCapturing((cudaStream_t)stream, &cap);
+  if (ce == cudaSuccess && cap != cudaStreamCaptureStatusNone) ce = cudaErrorStreamCaptureUnsupported;
+  if (ce != cudaSuccess) return wf_cuda_fail(ce, "wf_eval_any");
   void* scr = nullptr;
   char* work = nullptr;
   wf_status rs = wf_alloc(h, &scr, (size_t)B * vsz * (f64 ? sizeof(double2) : sizeof(float2)), "wf_eval_any scratch");
@@ -698,11 +702,12 @@ extern "C" wf_status wf_eval_any(wf_handle* h, int B, int C, int ny, int nx, int
     cudaStream_t st = (cudaStream_t)stream;
     cudaError_t e = f64 ? wf_any_launch<double>(G, d, mask, Ninv, P, s, grad, chi2, scr, work, st)
                         : wf_any_launch<float>(G, d, mask, Ninv, P, s, grad, chi2, scr, work, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    const cudaError_t es = cudaStreamSynchronize(st);  // also after a failed launch: earlier ones may still run
+    if (e == cudaSuccess) e = es;
     if (e != cudaSuccess) rs = wf_cuda_fail(e, "wf_eval_any");
   }
-  wf_free(h, work);
-  wf_free(h, scr);
+  wf_free_idle(h, work);
+  wf_free_idle(h, scr);
   return rs;
 }
 

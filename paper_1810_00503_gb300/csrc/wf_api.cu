@@ -199,6 +199,33 @@ static void wf_make_twiddles_all(double2* out) {
   }
 }
 
+// The handle's memory pool; without one (no pool support) it allocates plainly.
+static void pool_create(wf_handle* h) {
+  cudaMemPoolProps pr;
+  memset(&pr, 0, sizeof pr);
+  pr.allocType = cudaMemAllocationTypePinned;
+  pr.location.type = cudaMemLocationTypeDevice;
+  pr.location.id = h->device;
+  if (cudaStreamCreateWithFlags(&h->pool_stream, cudaStreamNonBlocking) != cudaSuccess) {
+    h->pool_stream = nullptr;
+  } else if (cudaMemPoolCreate(&h->pool, &pr) != cudaSuccess) {
+    h->pool = nullptr;
+  } else {
+    unsigned long long keep = h->limit ? 0 : WF_POOL_KEEP;
+    cudaMemPoolSetAttribute(h->pool, cudaMemPoolAttrReleaseThreshold, &keep);
+  }
+  cudaGetLastError();
+}
+// Which allocations come from it.  Larger ones gain nothing that matters beside the
+// work they are for, and take 3 ms more to map for a history ring of 10 GB.
+static bool pooled(const wf_handle* h, size_t bytes) { return h->pool && bytes <= WF_POOL_ONE; }
+static void pool_destroy(wf_handle* h) {
+  if (h->pool_stream) cudaStreamSynchronize(h->pool_stream);
+  if (h->pool) cudaMemPoolDestroy(h->pool);
+  if (h->pool_stream) cudaStreamDestroy(h->pool_stream);
+  for (auto& q : h->pinned) cudaFreeHost(q.first);
+}
+
 extern "C" wf_status wf_create(wf_handle** out, size_t workspace_limit) {
   if (!out) return wf_fail(WF_EINVAL, "wf_create: null output pointer");
   *out = nullptr;
@@ -206,13 +233,17 @@ extern "C" wf_status wf_create(wf_handle** out, size_t workspace_limit) {
   if (!h) return wf_fail(WF_ENOMEM, "wf_create: host allocation failed");
   h->limit = workspace_limit;
   h->used = 0;
+  h->pool = nullptr;
+  h->pool_stream = nullptr;
   cudaError_t e = cudaGetDevice(&h->device);
   if (e != cudaSuccess) { delete h; return wf_cuda_fail(e, "wf_create: cudaGetDevice"); }
+  pool_create(h);
   double2* tw64 = (double2*)malloc(sizeof(double2) * WF_TWTAB_ALL);
   float2* tw32 = (float2*)malloc(sizeof(float2) * WF_TWTAB_ALL);
   if (!tw64 || !tw32) {
     free(tw64);
     free(tw32);
+    pool_destroy(h);
     delete h;
     return wf_fail(WF_ENOMEM, "wf_create: host allocation failed");
   }
@@ -233,6 +264,7 @@ extern "C" wf_status wf_create(wf_handle** out, size_t workspace_limit) {
   if (s != WF_OK || e != cudaSuccess) {
     wf_free(h, h->tw64);
     wf_free(h, h->tw32);
+    pool_destroy(h);
     delete h;
     return s != WF_OK ? s : wf_cuda_fail(e, "wf_create: twiddle tables");
   }
@@ -244,6 +276,7 @@ extern "C" wf_status wf_destroy(wf_handle* h) {
   if (!h) return WF_OK;
   wf_free(h, h->tw64);
   wf_free(h, h->tw32);
+  pool_destroy(h);
   delete h;
   return WF_OK;
 }
@@ -257,8 +290,9 @@ extern "C" wf_status wf_workspace_used(const wf_handle* h, size_t* bytes) {
 
 static void free_problem(wf_problem* p) {
   if (!p) return;
+  cudaDeviceSynchronize();
   void* ptrs[] = {p->d, p->w, p->sp, p->sp0, p->scratch, p->part, p->flags, p->bpart};
-  for (void* q : ptrs) wf_free(p->h, q);
+  for (void* q : ptrs) wf_free_idle(p->h, q);
   wf_solver_free(p);
   free(p);
 }
@@ -272,7 +306,19 @@ wf_status wf_alloc(wf_handle* h, void** ptr, size_t bytes, const char* what) {
                      bytes, h->used, h->limit);
     h->used += bytes;  // reserved before the allocation, so concurrent callers cannot overshoot
   }
-  cudaError_t e = cudaMalloc(ptr, bytes);
+  cudaError_t e;
+  if (pooled(h, bytes)) {
+    e = cudaMallocFromPoolAsync(ptr, bytes, h->pool, h->pool_stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(h->pool_stream);  // usable on every stream from here
+    if (e == cudaErrorMemoryAllocation) {  // once more without what the pool keeps
+      cudaGetLastError();
+      cudaMemPoolTrimTo(h->pool, 0);
+      e = cudaMallocFromPoolAsync(ptr, bytes, h->pool, h->pool_stream);
+      if (e == cudaSuccess) e = cudaStreamSynchronize(h->pool_stream);
+    }
+  } else {
+    e = cudaMalloc(ptr, bytes);
+  }
   if (e != cudaSuccess) {
     *ptr = nullptr;
     cudaGetLastError();
@@ -289,13 +335,50 @@ wf_status wf_alloc(wf_handle* h, void** ptr, size_t bytes, const char* what) {
 
 void wf_free(wf_handle* h, void* ptr) {
   if (!ptr) return;
-  cudaFree(ptr);
-  std::lock_guard<std::mutex> lock(h->mu);
-  auto it = h->live.find(ptr);
-  if (it != h->live.end()) {
-    h->used -= it->second;
-    h->live.erase(it);
+  cudaDeviceSynchronize();
+  wf_free_idle(h, ptr);
+}
+
+void wf_free_idle(wf_handle* h, void* ptr) {
+  if (!ptr) return;
+  size_t bytes = 0;
+  {
+    std::lock_guard<std::mutex> lock(h->mu);
+    auto it = h->live.find(ptr);
+    if (it != h->live.end()) {
+      bytes = it->second;
+      h->live.erase(it);
+    }
   }
+  if (pooled(h, bytes)) cudaFreeAsync(ptr, h->pool_stream);
+  else cudaFree(ptr);
+  std::lock_guard<std::mutex> lock(h->mu);
+  h->used -= bytes;
+}
+
+cudaError_t wf_pinned_alloc(wf_handle* h, void** ptr, size_t bytes) {
+  {
+    std::lock_guard<std::mutex> lock(h->mu);
+    for (size_t i = 0; i < h->pinned.size(); ++i)
+      if (h->pinned[i].second == bytes) {
+        *ptr = h->pinned[i].first;
+        h->pinned.erase(h->pinned.begin() + i);
+        return cudaSuccess;
+      }
+  }
+  return cudaMallocHost(ptr, bytes);
+}
+
+void wf_pinned_free(wf_handle* h, void* ptr, size_t bytes) {
+  if (!ptr) return;
+  {
+    std::lock_guard<std::mutex> lock(h->mu);
+    if (h->pinned.size() < WF_PINNED_KEEP) {
+      h->pinned.emplace_back(ptr, bytes);
+      return;
+    }
+  }
+  cudaFreeHost(ptr);
 }
 
 extern "C" wf_status wf_problem_create_rect(wf_handle* h, const wf_map* maps, int count, int ny, int nx, int C,
@@ -366,10 +449,10 @@ extern "C" wf_status wf_problem_create_rect(wf_handle* h, const wf_map* maps, in
   if (e == cudaSuccess) {
     if (precision == WF_FP64)
       e = wf_launch_prep<double>(p->g, dp, mp, np, pp, dtype == WF_F64, count, p->d, p->w, p->sp,
-                                 shared, p->flags, st);
+                                 shared, p->flags, p->part, st);
     else
       e = wf_launch_prep<float>(p->g, dp, mp, np, pp, dtype == WF_F64, count, p->d, p->w, p->sp,
-                                shared, p->flags, st);
+                                shared, p->flags, p->part, st);
   }
   free(dp);
   if (e != cudaSuccess) { free_problem(p); return wf_cuda_fail(e, "wf_problem_create: input preparation"); }

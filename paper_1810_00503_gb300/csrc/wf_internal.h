@@ -286,7 +286,8 @@ enum { WF_IN_PK = 0, WF_IN_STD = 1 };
 template <typename T>
 cudaError_t wf_launch_prep(const WfGeo& g, const void* const* dptr, const unsigned char* const* mptr,
                            const void* const* nptr, const void* const* pptr, int in_f64, int B,
-                           void* d, void* w, void* sp, int sp_shared, int* flags, cudaStream_t st);
+                           void* d, void* w, void* sp, int sp_shared, int* flags,
+                           void* work /* 32 bytes a map */, cudaStream_t st);
 template <typename T>
 cudaError_t wf_launch_set_data(const WfGeo& g, const void* src, int B, void* d, cudaStream_t st);
 template <typename T>

@@ -203,14 +203,12 @@ inline int grid1d(size_t total, int cap) {
   cudaError_t wf_launch_prep(const WfGeo& g, const void* const* dptr,
                                 const unsigned char* const* mptr, const void* const* nptr,
                                 const void* const* pptr, int in_f64, int B, void* d, void* w,
-                                void* sp, int sp_shared, int* flags, cudaStream_t st) {
+                                void* sp, int sp_shared, int* flags, void* work, cudaStream_t st) {
     WfMapPtrs* hm = (WfMapPtrs*)malloc(sizeof(WfMapPtrs) * (size_t)B);
     if (!hm) return cudaErrorMemoryAllocation;
     for (int i = 0; i < B; ++i) hm[i] = WfMapPtrs{dptr[i], mptr[i], nptr[i], pptr[i]};
-    WfMapPtrs* dm = nullptr;
-    cudaError_t e = cudaMallocAsync((void**)&dm, sizeof(WfMapPtrs) * (size_t)B, st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(dm, hm, sizeof(WfMapPtrs) * (size_t)B,
-                                              cudaMemcpyHostToDevice, st);
+    WfMapPtrs* dm = (WfMapPtrs*)work;
+    cudaError_t e = cudaMemcpyAsync(dm, hm, sizeof(WfMapPtrs) * (size_t)B, cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) {
       const size_t npix = (size_t)g.C * g.n * g.nx;
       k_prep<T><<<dim3(wfimpl::grid1d(npix, 1024), B), 256, 0, st>>>(g, dm, in_f64, (T*)d, (T*)w,
@@ -218,7 +216,6 @@ inline int grid1d(size_t total, int cap) {
       e = cudaGetLastError();
     }
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    if (dm) cudaFreeAsync(dm, st);
     free(hm);
     return e;
   }
@@ -361,7 +358,7 @@ cudaError_t wf_launch_eval_pk(const WfGeo& g, const WfBufs& b, const void* src, 
   template cudaError_t wf_launch_prep<T>(const WfGeo&, const void* const*,                         \
                                          const unsigned char* const*, const void* const*,          \
                                          const void* const*, int, int, void*, void*, void*, int,   \
-                                         int*, cudaStream_t);                                      \
+                                         int*, void*, cudaStream_t);                                      \
   template cudaError_t wf_launch_set_data<T>(const WfGeo&, const void*, int, void*, cudaStream_t); \
   template cudaError_t wf_launch_eval<T>(const WfGeo&, const WfBufs&, int, int, const void*,       \
                                          void*, double*, cudaStream_t);                            \

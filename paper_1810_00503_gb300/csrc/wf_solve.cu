@@ -569,10 +569,11 @@ void wf_solver_free(wf_problem* p) {
   if (S->exec) cudaGraphExecDestroy(S->exec);
   void* ptrs[] = {S->s, S->g, S->ring, S->st, S->nact, S->stats_dev, S->hist, S->r_s64, S->r_g64, S->r_d64,
                   S->r_w64, S->r_sp64, S->r_scr64, S->r_res};
-  for (void* q : ptrs) wf_free(p->h, q);
+  cudaDeviceSynchronize();
+  for (void* q : ptrs) wf_free_idle(p->h, q);
   if (S->r_res_host) cudaFreeHost(S->r_res_host);
-  if (S->nact_host) cudaFreeHost(S->nact_host);
-  if (S->stats_host) cudaFreeHost(S->stats_host);
+  wf_pinned_free(p->h, S->nact_host, sizeof(int));
+  wf_pinned_free(p->h, S->stats_host, sizeof(double) * 5 * S->B);
   if (S->stream) cudaStreamDestroy(S->stream);
   if (S->ev_in) cudaEventDestroy(S->ev_in);
   if (S->ev_out) cudaEventDestroy(S->ev_out);
@@ -596,8 +597,8 @@ static wf_status ensure_solver(wf_problem* p, int m) {
   if (s == WF_OK) s = wf_alloc(p->h, (void**)&S->nact, sizeof(int), "active counter");
   if (s == WF_OK) s = wf_alloc(p->h, (void**)&S->stats_dev, sizeof(double) * 5 * p->count, "statistics");
   cudaError_t e = cudaSuccess;
-  if (s == WF_OK) e = cudaMallocHost((void**)&S->nact_host, sizeof(int));
-  if (s == WF_OK && e == cudaSuccess) e = cudaMallocHost((void**)&S->stats_host, sizeof(double) * 5 * p->count);
+  if (s == WF_OK) e = wf_pinned_alloc(p->h, (void**)&S->nact_host, sizeof(int));
+  if (s == WF_OK && e == cudaSuccess) e = wf_pinned_alloc(p->h, (void**)&S->stats_host, sizeof(double) * 5 * p->count);
   if (s == WF_OK && e == cudaSuccess) e = cudaStreamCreateWithFlags(&S->stream, cudaStreamNonBlocking);
   if (s == WF_OK && e == cudaSuccess) e = cudaEventCreateWithFlags(&S->ev_in, cudaEventDisableTiming);
   if (s == WF_OK && e == cudaSuccess) e = cudaEventCreateWithFlags(&S->ev_out, cudaEventDisableTiming);

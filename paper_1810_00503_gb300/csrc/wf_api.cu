@@ -61,13 +61,13 @@ static void wf_geo_tiles(WfGeo& g, int tc_div, int rb_div) {
   g.RB = rb;
   g.nrb = g.C * g.n / rb;
   if (g.colinv_kind == WF_COLINV_REG_K) {
-    int tc = wf_rg_tc(g.n, g.C, tc_div);
+    int tc = wf_rg_tc(g.n, g.C, tc_div, g.f64);
     while ((g.h + tc - 1) / tc > g.maxblk) tc *= 2;
     g.TC = tc;
     g.ntile = (g.h + tc - 1) / tc;  // one tile, partly empty, where it is wider than the map
   }
   if (g.row_kind == WF_ROW_REG_K) {  // eight warps a block, or 1/2 and 1/4 of them
-    const int per = wf_rg_rows(g.nx), need = (g.C * g.n + per - 1) / per;
+    const int per = wf_rg_rows(g.nx, g.f64), need = (g.C * g.n + per - 1) / per;
     int warps = 8 / rb_div;
     while (warps > need) warps /= 2;
     while (warps < 8 && (need + warps - 1) / warps > g.maxblk) warps *= 2;
@@ -88,8 +88,9 @@ static void wf_geo_fix_kind(WfGeo& g) {
   }
 }
 
-WfGeo wf_make_geo(int ny, int nx, int C, int B) {
+WfGeo wf_make_geo(int ny, int nx, int C, int B, bool f64) {
   WfGeo g;
+  g.f64 = f64;
   g.n = ny;
   g.nx = nx;
   g.h = nx / 2;
@@ -117,7 +118,7 @@ WfGeo wf_make_geo(int ny, int nx, int C, int B) {
   wf_geo_tiles(g, WF_TUNE_MAXDIV, WF_TUNE_MAXDIV);
   g.maxblk = g.ntile > g.nrb ? g.ntile : g.nrb;
   if (g.ncomb > g.maxblk) g.maxblk = g.ncomb;
-  const int wide = wf_rg_tc(ny, C, 1), tiles = (g.h + wide - 1) / wide;
+  const int wide = wf_rg_tc(ny, C, 1, f64), tiles = (g.h + wide - 1) / wide;
   if (tiles > g.maxblk) g.maxblk = tiles;
   g.colinv_kind = WF_COLINV_REG_K;
   g.row_kind = WF_ROW_REG_K;
@@ -125,8 +126,8 @@ WfGeo wf_make_geo(int ny, int nx, int C, int B) {
   return g;
 }
 
-WfGeo wf_make_geo_pass(int ny, int nx, int C, int B) {
-  WfGeo g = wf_make_geo(ny, nx, C, B);
+WfGeo wf_make_geo_pass(int ny, int nx, int C, int B, bool f64) {
+  WfGeo g = wf_make_geo(ny, nx, C, B, f64);
   const int fill = 2 * WF_SMS;  // two blocks per SM
   int tc_div = 1, rb_div = 1;
   while (tc_div < WF_TUNE_MAXDIV && (long long)B * g.ntile < fill) wf_geo_tiles(g, tc_div *= 2, rb_div);
@@ -417,8 +418,8 @@ extern "C" wf_status wf_problem_create_rect(wf_handle* h, const wf_map* maps, in
   p->dtype = dtype;
   p->precision = precision;
   p->m = lbfgs_m;
-  p->g = wf_make_geo(ny, nx, C, count);
-  p->gp = wf_make_geo_pass(ny, nx, C, count);
+  p->g = wf_make_geo(ny, nx, C, count, precision == WF_FP64);
+  p->gp = wf_make_geo_pass(ny, nx, C, count, precision == WF_FP64);
   p->elt = precision == WF_FP64 ? sizeof(double) : sizeof(float);
   int shared = 1;
   for (int i = 1; i < count; ++i) shared &= maps[i].P == maps[0].P;

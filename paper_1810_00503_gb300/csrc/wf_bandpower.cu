@@ -327,7 +327,7 @@ extern "C" wf_status bandpower_estimate_rect(wf_handle* h, const wf_map* data, i
   Scope sc(h);
   // Theta_fid and the band-restricted power tables
   double* theta = nullptr;  // then the work space of its sums
-  const WfGeo geo = wf_make_geo(ny, nx, C, 1);
+  const WfGeo geo = wf_make_geo(ny, nx, C, 1, dtype == WF_F64);
   BP_OK(wf_alloc(h, (void**)&theta, sizeof(double) * nb * (1 + 2 * (size_t)wf_band_nblk(geo)), "theta_fid"));
   sc.add(theta);
   if (dtype == WF_F64) BP_TRY(wf_launch_theta_fid<double>(geo, data->P, in->band, nb, theta + nb, theta, st));

@@ -233,27 +233,30 @@ struct WfGeo {
   int maxblk;      // stride of the partial-sum slots: covers every tile choice
   int colinv_kind, row_kind;  // WF_COLINV_*_K, WF_ROW_*_K
   int tc_div, rb_div;         // TC and RB are the widest tile divided by these (1, 2, 4)
+  bool f64;                   // working type: FP64 sequences of 512 take twice the threads (wf_reg.cuh)
   int col_plan, row_plan;     // radix plan of the TMA-fed stage's passes; row_plan is carried only (0..WF_NPLAN-1)
 };
 
 // The register-resident stages (wf_reg.cuh) with their widest tiles; B: maps per
 // launch, which sets the streaming kernels' chunk groups (0: many).
-WfGeo wf_make_geo(int ny, int nx, int C, int B);
+WfGeo wf_make_geo(int ny, int nx, int C, int B, bool f64);
 // The same with tiles narrowed for a batch too small to fill the chip with the
 // widest: what the objective's passes run (the L-BFGS stages are tuned).
-WfGeo wf_make_geo_pass(int ny, int nx, int C, int B);
+WfGeo wf_make_geo_pass(int ny, int nx, int C, int B, bool f64);
 
 // Register-resident stages.  Widest tile: wf_rg_seq(N) sequences a block (256
 // threads from 64 rows up; 64-byte rows of a tile at 1024, 128-byte rows and
 // more below), and 1/2 and 1/4 of it.
-__host__ __device__ constexpr int wf_rg_seq(int N) { return N == 1024 ? 8 : N >= 256 ? 16 : 32; }
-__host__ __device__ constexpr int wf_rg_tc(int N, int C, int div) {
-  const int seq = N == 8 && div == 4 ? 16 : wf_rg_seq(N) / div;  // at least a warp a block
+__host__ __device__ constexpr int wf_rg_seq(int N, bool f64) {
+  return N == 1024 || (N == 512 && f64) ? 8 : N >= 256 ? 16 : 32;
+}
+__host__ __device__ constexpr int wf_rg_tc(int N, int C, int div, bool f64) {
+  const int seq = N == 8 && div == 4 ? 16 : wf_rg_seq(N, f64) / div;  // at least a warp a block
   return seq / C < 2 ? 2 : seq / C;
 }
 // Rows a warp of the row stage takes: pairs of rows, 32 or fewer values a thread.
-__host__ __device__ constexpr int wf_rg_rows(int nx) {
-  return nx == 1024 ? 2 : nx >= 256 ? 4 : nx >= 64 ? 8 : nx >= 16 ? 16 : 32;
+__host__ __device__ constexpr int wf_rg_rows(int nx, bool f64) {
+  return nx == 1024 || (nx == 512 && f64) ? 2 : nx >= 256 ? 4 : nx >= 64 ? 8 : nx >= 16 ? 16 : 32;
 }
 // Blocks per map of the band reductions: about 4096 modes each, at most 64.
 inline int wf_band_nblk(const WfGeo& g) {

@@ -37,7 +37,8 @@ k_multi_col(const __grid_constant__ WfMultiGrid r, const __grid_constant__ WfMul
       if constexpr (INV) wf_rg_lb_colinv_map<T, C, N, TC>(a.g[q], a.b[q], a.lb[q], kb.y, kb.x);
       else wf_rg_lb_colfwd_map<T, C, N, TC>(a.g[q], a.b[q], a.lb[q], kb.y, kb.x);
     };
-    constexpr int A = wf_rg_tc(N, C, 1), B = wf_rg_tc(N, C, 2);
+    constexpr bool F64 = sizeof(T) == 8;
+    constexpr int A = wf_rg_tc(N, C, 1, F64), B = wf_rg_tc(N, C, 2, F64);
     if (a.g[q].TC == A) width(std::integral_constant<int, A>());
     else width(std::integral_constant<int, B>());
   });
@@ -47,17 +48,18 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 2 : 1)
 k_multi_row(const __grid_constant__ WfMultiGrid r, const __grid_constant__ WfMultiArgs a) {
   WfBlk kb;
   const int q = wf_multi_block(r, kb);
-  if ((int)threadIdx.x >= 32 * (a.g[q].RB / wf_rg_rows(a.g[q].nx))) return;
+  if ((int)threadIdx.x >= 32 * (a.g[q].RB / wf_rg_rows(a.g[q].nx, sizeof(T) == 8))) return;
   wf_rg_switch(a.g[q].nx, [&](auto n) { wf_rg_lb_row_map<T, decltype(n)::value>(a.g[q], a.b[q], a.lb[q], kb.y, kb.x); });
 }
 
 // Shared memory of a problem's stages.
 template <typename T> inline size_t wf_multi_col_smem(const WfGeo& g) {
+  constexpr bool F64 = sizeof(T) == 8;
   size_t sm = 0;
   wfimpl::rg_length(g.n, [&](auto n) {
-    const bool wide = g.TC == wf_rg_tc(n(), g.C, 1);
-    if (g.C == 1) sm = wide ? WfRegCol<T, 1, n(), wf_rg_tc(n(), 1, 1)>::SMEM : WfRegCol<T, 1, n(), wf_rg_tc(n(), 1, 2)>::SMEM;
-    else sm = wide ? WfRegCol<T, 2, n(), wf_rg_tc(n(), 2, 1)>::SMEM : WfRegCol<T, 2, n(), wf_rg_tc(n(), 2, 2)>::SMEM;
+    const bool wide = g.TC == wf_rg_tc(n(), g.C, 1, F64);
+    if (g.C == 1) sm = wide ? WfRegCol<T, 1, n(), wf_rg_tc(n(), 1, 1, F64)>::SMEM : WfRegCol<T, 1, n(), wf_rg_tc(n(), 1, 2, F64)>::SMEM;
+    else sm = wide ? WfRegCol<T, 2, n(), wf_rg_tc(n(), 2, 1, F64)>::SMEM : WfRegCol<T, 2, n(), wf_rg_tc(n(), 2, 2, F64)>::SMEM;
     return cudaSuccess;
   });
   return sm;
@@ -65,7 +67,7 @@ template <typename T> inline size_t wf_multi_col_smem(const WfGeo& g) {
 template <typename T> inline size_t wf_multi_row_smem(const WfGeo& g) {
   size_t sm = 0;
   wfimpl::rg_length(g.nx, [&](auto n) {
-    sm = WfRegRow<T, n()>::smem(g.RB / wf_rg_rows(g.nx));
+    sm = WfRegRow<T, n()>::smem(g.RB / wf_rg_rows(g.nx, sizeof(T) == 8));
     return cudaSuccess;
   });
   return sm;
@@ -82,7 +84,7 @@ cudaError_t wf_launch_multi_fft(const WfMultiArgs& a, int stage, cudaStream_t st
     if (s > sm) sm = s;
   }
   auto k = row ? k_multi_row<T> : stage == 0 ? k_multi_col<T, C, true> : k_multi_col<T, C, false>;
-  cudaError_t e = wfimpl::ensure_smem(k, WfRegCol<T, 1, 1024, wf_rg_tc(1024, 1, 1)>::SMEM, &done[stage]);  // the largest
+  cudaError_t e = wfimpl::ensure_smem(k, WfRegCol<T, 1, 1024, wf_rg_tc(1024, 1, 1, sizeof(T) == 8)>::SMEM, &done[stage]);  // the largest
   if (e != cudaSuccess) return e;
   k<<<r.start[a.np], 256, sm, st>>>(r, a);
   return cudaGetLastError();

@@ -77,7 +77,7 @@ __global__ void k_noalloc_sqrtp(const T* P, size_t total, int n, T* sp) {
 template <typename T>
 static wf_status noalloc_impl(unsigned char* base, const void* s, const void* d, const void* w, const void* P,
                               int n, int C, int count, double* chi2, void* grad, cudaStream_t st) {
-  const WfGeo g = wf_make_geo_pass(n, n, C, count);
+  const WfGeo g = wf_make_geo_pass(n, n, C, count, sizeof(T) == 8);
   const size_t elt = sizeof(T);
   const size_t nsp = (size_t)C * n * (n / 2 + 1);
   const size_t off_sp = WF_NOALLOC_DATA;

@@ -42,6 +42,18 @@ template <> struct WfReg<64> { static constexpr int NV = 8, RA = 8, RB = 8; };
 template <> struct WfReg<32> { static constexpr int NV = 8, RA = 4, RB = 8; };
 template <> struct WfReg<16> { static constexpr int NV = 4, RA = 4, RB = 4; };
 template <> struct WfReg<8> { static constexpr int NV = 4, RA = 2, RB = 4; };
+// Passes in the working type: R1, R2 of the column and the forward row transforms,
+// I1, I2 of the inverse row transform (the radices the other way round).  FP64 at
+// 512 holds 16 values a thread and splits the radix-32 butterflies of pass 2 over
+// two threads: a warp's FP64 instruction holds its unit for 64 cycles, so a map's
+// time is that of one warp's instructions until every unit has a warp, and 32
+// values a thread make only 128 warps of a 512^2 map.  One map of 512^2, the
+// objective pass: 186 -> 111 us.  It costs nothing where
+// the chip is full (40 maps: 1.65 -> 1.60 ms).
+template <typename T, int N> struct WfRegT {
+  static constexpr int NV = WfReg<N>::NV, R1 = WfReg<N>::RB, R2 = WfReg<N>::RA, I1 = R2, I2 = R1;
+};
+template <> struct WfRegT<double, 512> { static constexpr int NV = 16, R1 = 16, R2 = 32, I1 = 16, I2 = 32; };
 
 __device__ __forceinline__ float wf_fma(float a, float b, float c) { return fmaf(a, b, c); }
 __device__ __forceinline__ double wf_fma(double a, double b, double c) { return fma(a, b, c); }
@@ -126,7 +138,7 @@ template <typename T, int S, int R2> struct WfXch {
 template <typename T, int N, int R1, int R2, int NV, int DIR, int PITCH, int S>
 __device__ __forceinline__ void wf_rg_pass1(V2<T>* v, V2<T>* sm, const V2<T>* tw, int g) {
   constexpr int G = N / NV, NB = NV / R1;
-  static_assert(R1 * R2 == N && NV % R1 == 0 && NV % R2 == 0, "passes");
+  static_assert(R1 * R2 == N && NV % R1 == 0 && (NV % R2 == 0 || R2 == 2 * NV), "passes");
 #pragma unroll
   for (int i = 0; i < NB; ++i) {
     wf_rg_dft<T, R1, DIR, NB>(v + i);
@@ -136,23 +148,46 @@ __device__ __forceinline__ void wf_rg_pass1(V2<T>* v, V2<T>* sm, const V2<T>* tw
     for (int q = 1; q < R1; ++q) sm[q * PITCH + j * S] = cmul<T>(v[i + q * NB], twid<T, DIR>(tw, q * R2 + j));
   }
 }
-// Place of the exchange that a thread's value m of pass 2 is read from.
+// Place of the exchange that a thread's value m of pass 2 is read from (a split
+// butterfly's two threads read both halves: this thread's half).
 template <int N, int R2, int NV, int PITCH, int S>
 __device__ __forceinline__ int wf_rg_place(int g, int m) {
-  constexpr int G = N / NV, NB = NV / R2;
-  return (g + G * (m % NB)) * PITCH + (m / NB) * S;
+  if constexpr (R2 > NV) {
+    constexpr int R1 = N / R2;
+    return (g & (R1 - 1)) * PITCH + (m + NV * (g / R1)) * S;
+  } else {
+    constexpr int G = N / NV, NB = NV / R2;
+    return (g + G * (m % NB)) * PITCH + (m / NB) * S;
+  }
 }
-// Read of the exchange, and pass 2.
-template <typename T, int N, int R1, int R2, int NV, int PITCH, int S>
-__device__ __forceinline__ void wf_rg_read(V2<T>* v, const V2<T>* sm, int g) {
+// Read of the exchange.  A butterfly of R2 = 2 NV values is split over the threads
+// q and q + R1: they form y_j + y_{j+NV} and (y_j - y_{j+NV}) w^j, whose length-NV
+// transforms are the outputs of even and odd index, elements g + G k of both.
+template <typename T, int N, int R1, int R2, int NV, int DIR, int PITCH, int S>
+__device__ __forceinline__ void wf_rg_read(V2<T>* v, const V2<T>* sm, const V2<T>* tw, int g) {
+  if constexpr (R2 > NV) {
+    const V2<T>* y = sm + (g & (R1 - 1)) * PITCH;
+    if (g < R1) {
 #pragma unroll
-  for (int m = 0; m < NV; ++m) v[m] = sm[wf_rg_place<N, R2, NV, PITCH, S>(g, m)];
+      for (int m = 0; m < NV; ++m) v[m] = cadd<T>(y[m * S], y[(m + NV) * S]);
+    } else {  // w^j = the pass-1 root of (q, j) = (j, R1)
+#pragma unroll
+      for (int m = 0; m < NV; ++m) v[m] = cmul<T>(csub<T>(y[m * S], y[(m + NV) * S]), twid<T, DIR>(tw, m * R2 + R1));
+    }
+  } else {
+#pragma unroll
+    for (int m = 0; m < NV; ++m) v[m] = sm[wf_rg_place<N, R2, NV, PITCH, S>(g, m)];
+  }
 }
 template <typename T, int N, int R1, int R2, int NV, int DIR>
 __device__ __forceinline__ void wf_rg_pass2(V2<T>* v) {
-  constexpr int NB = NV / R2;
+  if constexpr (R2 > NV) {  // half a butterfly (wf_rg_read has done its first step)
+    wf_rg_dft<T, NV, DIR, 1>(v);
+  } else {
+    constexpr int NB = NV / R2;
 #pragma unroll
-  for (int i = 0; i < NB; ++i) wf_rg_dft<T, R2, DIR, NB>(v + i);
+    for (int i = 0; i < NB; ++i) wf_rg_dft<T, R2, DIR, NB>(v + i);
+  }
 }
 
 // Pass-1 twiddles of a length-N transform with radices R1, R2 into shared
@@ -199,8 +234,8 @@ template <typename T, int NV> __host__ __device__ constexpr int wf_rg_minb(int t
 // the map (h < TC) has idle columns: they load the last one and store nothing.
 // ---------------------------------------------------------------------------
 template <typename T, int C, int N, int TC> struct WfRegCol {
-  static constexpr int NV = WfReg<N>::NV, G = N / NV, S = C * TC, THREADS = S * G;
-  static constexpr int R1 = WfReg<N>::RB, R2 = WfReg<N>::RA;  // larger radix first
+  static constexpr int NV = WfRegT<T, N>::NV, G = N / NV, S = C * TC, THREADS = S * G;
+  static constexpr int R1 = WfRegT<T, N>::R1, R2 = WfRegT<T, N>::R2;
   static constexpr int PITCH = WfXch<T, S, R2>::PITCH;
   static constexpr size_t XCH = (size_t)R1 * PITCH;            // values of the exchange buffer
   static constexpr size_t SMEM = (XCH + N) * sizeof(V2<T>);    // and the twiddles
@@ -296,7 +331,7 @@ __device__ __forceinline__ void wf_rg_cols(V2<T>* v, V2<T>* xch_t, const V2<T>* 
   __syncthreads();  // twiddles staged; an earlier exchange has been read
   wf_rg_pass1<T, N, K::R1, K::R2, K::NV, DIR, K::PITCH, K::S>(v, xch_t, s_tw, g);
   __syncthreads();
-  wf_rg_read<T, N, K::R1, K::R2, K::NV, K::PITCH, K::S>(v, xch_t, g);
+  wf_rg_read<T, N, K::R1, K::R2, K::NV, DIR, K::PITCH, K::S>(v, xch_t, s_tw, g);
 }
 
 // Inverse column stage of the tile at packed column kx0: spectrum (packed or
@@ -386,7 +421,8 @@ __device__ __forceinline__ void wf_rg_colfwd_front(V2<T>* v, const WfGeo& geo, c
   wf_rg_cols<T, C, N, TC, -1>(v, xch + t, s_tw, g);
   const unsigned a0 = (unsigned)(c * N + g) * pitch + (unsigned)kx, astep = K::G * pitch;
   auto fetch = [&]() {
-    __syncwarp();
+    if constexpr (K::R2 > K::NV) __syncthreads();  // two threads read a value
+    else __syncwarp();
 #pragma unroll
     for (int m = 0; m < K::NV; ++m)
       wf_cp_async<T>(xch + t + wf_rg_place<N, K::R2, K::NV, K::PITCH, K::S>(g, m),
@@ -553,13 +589,14 @@ __device__ __forceinline__ void wf_rg_lb_colfwd(const WfGeo& geo, const V2<T>* P
 // values in registers, r2c from there, store.
 // ---------------------------------------------------------------------------
 template <typename T, int NX> struct WfRegRow {
-  static constexpr int NV = WfReg<NX>::NV, G = NX / NV, SEQ = 32 / G, RA = WfReg<NX>::RA, RB = WfReg<NX>::RB;
-  static constexpr int PI = WfXch<T, 1, RB>::PITCH, PF = WfXch<T, 1, RA>::PITCH;  // inverse (RA, RB), forward (RB, RA)
-  static constexpr int XI = RA * PI, XF = RB * PF, XM = XI > XF ? XI : XF;
+  static constexpr int NV = WfRegT<T, NX>::NV, G = NX / NV, SEQ = 32 / G;
+  static constexpr int I1 = WfRegT<T, NX>::I1, I2 = WfRegT<T, NX>::I2, F1 = WfRegT<T, NX>::R1, F2 = WfRegT<T, NX>::R2;
+  static constexpr int PI = WfXch<T, 1, I2>::PITCH, PF = WfXch<T, 1, F2>::PITCH;  // inverse, forward
+  static constexpr int XI = I1 * PI, XF = F1 * PF, XM = XI > XF ? XI : XF;
   // a sequence's exchange places; the sequences of a half-warp sit G values apart
   // modulo 16
   static constexpr int XCH = G >= 16 ? XM : (XM + 15) / 16 * 16 + G;
-  static constexpr int NTW = RA == RB ? NX : 2 * NX;  // twiddles of both directions
+  static constexpr int NTW = I1 == F1 ? NX : 2 * NX;  // twiddles of both directions
   static constexpr size_t smem(int warps) { return ((size_t)warps * SEQ * XCH + NTW) * sizeof(V2<T>); }
 };
 
@@ -568,15 +605,16 @@ __device__ __forceinline__ void wf_rg_row_fft(V2<T>* v, V2<T>* xch, const V2<T>*
   typedef WfRegRow<T, NX> K;
   __syncwarp();  // an earlier exchange has been read
   if constexpr (DIR > 0) {
-    wf_rg_pass1<T, NX, K::RA, K::RB, K::NV, DIR, K::PI, 1>(v, xch, s_tw, g);
+    wf_rg_pass1<T, NX, K::I1, K::I2, K::NV, DIR, K::PI, 1>(v, xch, s_tw, g);
     __syncwarp();
-    wf_rg_read<T, NX, K::RA, K::RB, K::NV, K::PI, 1>(v, xch, g);
-    wf_rg_pass2<T, NX, K::RA, K::RB, K::NV, DIR>(v);
+    wf_rg_read<T, NX, K::I1, K::I2, K::NV, DIR, K::PI, 1>(v, xch, s_tw, g);
+    wf_rg_pass2<T, NX, K::I1, K::I2, K::NV, DIR>(v);
   } else {
-    wf_rg_pass1<T, NX, K::RB, K::RA, K::NV, DIR, K::PF, 1>(v, xch, s_tw + (K::RA == K::RB ? 0 : NX), g);
+    const V2<T>* tw = s_tw + (K::I1 == K::F1 ? 0 : NX);
+    wf_rg_pass1<T, NX, K::F1, K::F2, K::NV, DIR, K::PF, 1>(v, xch, tw, g);
     __syncwarp();
-    wf_rg_read<T, NX, K::RB, K::RA, K::NV, K::PF, 1>(v, xch, g);
-    wf_rg_pass2<T, NX, K::RB, K::RA, K::NV, DIR>(v);
+    wf_rg_read<T, NX, K::F1, K::F2, K::NV, DIR, K::PF, 1>(v, xch, tw, g);
+    wf_rg_pass2<T, NX, K::F1, K::F2, K::NV, DIR>(v);
   }
 }
 
@@ -639,13 +677,13 @@ __device__ __forceinline__ void wf_rg_row(const WfGeo& geo, V2<T>* scratch, cons
   {
     const V2<T>* roots = (const V2<T>*)tw_;
     if constexpr (MODE != WF_ROW_RFFT) {
-      for (int i = threadIdx.x; i < NX; i += nth) s_tw[i] = roots[((i / K::RB) * (i % K::RB)) * (WF_NT / NX)];
+      for (int i = threadIdx.x; i < NX; i += nth) s_tw[i] = roots[((i / K::I2) * (i % K::I2)) * (WF_NT / NX)];
     }
-    if constexpr (K::RA != K::RB && (MODE == WF_ROW_RFFT || MODE == WF_ROW_DATA || MODE == WF_ROW_NODATA)) {
+    if constexpr (K::I1 != K::F1 && (MODE == WF_ROW_RFFT || MODE == WF_ROW_DATA || MODE == WF_ROW_NODATA)) {
       for (int i = threadIdx.x; i < NX; i += nth)
-        s_tw[NX + i] = roots[((i / K::RA) * (i % K::RA)) * (WF_NT / NX)];
+        s_tw[NX + i] = roots[((i / K::F2) * (i % K::F2)) * (WF_NT / NX)];
     } else if constexpr (MODE == WF_ROW_RFFT) {
-      for (int i = threadIdx.x; i < NX; i += nth) s_tw[i] = roots[((i / K::RA) * (i % K::RA)) * (WF_NT / NX)];
+      for (int i = threadIdx.x; i < NX; i += nth) s_tw[i] = roots[((i / K::F2) * (i % K::F2)) * (WF_NT / NX)];
     }
   }
   if constexpr (MODE == WF_ROW_DATA || MODE == WF_ROW_NODATA || MODE == WF_ROW_SIM) {
@@ -777,7 +815,7 @@ template <typename T, int NX>
 __device__ __forceinline__ void wf_rg_lb_row_map(const WfGeo& g, const WfBufs& b, const WfLbBufs& lb, int bm, int bx) {
   if (!lb.st[bm].active) return;
   wf_rg_row<T, WF_ROW_NODATA, NX>(g, (V2<T>*)b.scratch, nullptr, (const T*)b.w, nullptr, nullptr, b.part, b.tw, bm, bx,
-                                  g.RB / wf_rg_rows(NX));
+                                  g.RB / wf_rg_rows(NX, sizeof(T) == 8));
 }
 template <typename T, int C, int N, int TC>
 __device__ __forceinline__ void wf_rg_lb_colfwd_map(const WfGeo& g, const WfBufs& b, const WfLbBufs& lb, int bm, int bx) {

@@ -675,7 +675,7 @@ static bool variant_valid(int v) {
          b >= WF_ROW_REG_K && b <= WF_ROW_INPLACE_K && div_ok(c) && div_ok(d);
 }
 static WfGeo default_geo(const wf_problem* p) {
-  return wf_make_geo(p->n, p->nx, p->C, p->count);
+  return wf_make_geo(p->n, p->nx, p->C, p->count, p->precision == WF_FP64);
 }
 static WfGeo variant_geo(const WfGeo& base, int v) {
   return wf_geo_variant(base, (v / 1000) % 10, (v / 100) % 10, (v / 10) % 10, v % 10, v / 100000,

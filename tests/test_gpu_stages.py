@@ -22,7 +22,8 @@ TOL = {"fp64": 1e-12, "mixed": 2e-5}
 # (ny, nx, C, B): h = nx / 2 packed columns; the narrowing rule changes at
 # B * tiles = 304 (tiles of 8 columns at ny = 1024, 16 at 256 and 512, 32 below)
 SHAPES = [(8, 8, 2, 3), (8, 1024, 2, 1), (1024, 8, 1, 2), (16, 32, 1, 5), (32, 16, 2, 2), (64, 8, 1, 1),
-          (128, 16, 2, 3), (256, 32, 1, 40), (32, 64, 2, 160), (64, 128, 1, 161), (512, 64, 2, 77), (128, 256, 1, 76)]
+          (128, 16, 2, 3), (256, 32, 1, 40), (32, 64, 2, 160), (64, 128, 1, 161), (512, 64, 2, 77), (128, 256, 1, 76),
+          (64, 512, 2, 3), (512, 512, 1, 1)]
 
 
 @pytest.fixture(scope="module", autouse=True)

@@ -94,8 +94,8 @@ typedef struct {
   int refresh_every;  /* recompute the true gradient from the data every this many
                          iterations (0 = only at the start and the end); default 0 */
   int check_every;    /* iterations between host polls of the convergence flags
-                         (one synchronisation each); default 16 */
-  int use_graphs;     /* capture check_every iterations in one CUDA graph; default 1 */
+                         (one synchronisation each); default 16; max_iter bounds it */
+  int use_graphs;     /* capture the iterations between two polls in one CUDA graph; default 1 */
   void* stream;       /* cudaStream_t for all work of the call; NULL = default stream */
   int line_search;    /* wf_line_search; default WF_LS_EXACT */
   int pad_;
@@ -626,10 +626,11 @@ wf_status wf_eval_noalloc(const void* s, const void* d, const void* w, const voi
  *   P     [C][ny][nx/2+1]                   signal power per mode, >= 0, shared
  *   grad  like s, chi2 double [count]       outputs
  * Values are not checked.  Allocates its scratch (C ny (nx/2+1) complex per
- * map plus partial sums) from the handle, synchronises the stream and frees
- * it before returning.  Kernels: Stockham transforms with radix 4, 2, 3, 5 and
- * 7 passes in shared memory, one kernel per stage (inverse column, row,
- * forward column), partial sums added in a fixed order.
+ * map, partial sums, and tables of C ny (nx/2+1) values and both lengths' roots
+ * that the maps share) from the handle, synchronises the stream and frees it
+ * before returning.  Kernels: Stockham transforms of two to four passes with
+ * radices up to 16, one kernel per stage (tables, inverse column, row, forward
+ * column), partial sums added in a fixed order.
  * Errors: WF_EINVAL (null pointer, s == grad, count < 1, C not 1 or 2, a side
  * outside [2, 1024] or with a prime factor above 7, unknown precision),
  * WF_ENOMEM, WF_ECUDA. */

@@ -13,6 +13,7 @@
 //             the Gram matrices to give the next direction's coefficients.
 // Iterations are captured in CUDA graphs, `check_every` per graph; the host
 // reads one counter of active maps per graph launch.
+#include <algorithm>
 #include <math.h>
 #include <stdlib.h>
 #include <string.h>
@@ -865,20 +866,34 @@ static wf_status setup_args(wf_problem* p, WfSolver* S, const wf_opts* o) {
   return WF_OK;
 }
 
-// Capture `chunk` iterations in a CUDA graph on st (unless the graph in hand
-// was captured with the same settings).  Every kernel's attributes must have
-// been set outside capture: one plain iteration has run before.
+// Iterations between two polls, and of one graph: check_every, or all of a solve
+// of fewer.  Without the second bound a solve of few iterations runs its last
+// graph's remaining iterations on stopped maps, six launches that return at once
+// each (four FP64 maps of 64 x 1024, six iterations: 1086 -> 952 us).
+static int check_chunk(const wf_opts* o) {
+  const int chunk = o->check_every > 0 ? o->check_every : 16;
+  return o->max_iter < chunk ? o->max_iter : chunk;
+}
+// Iterations after which a solve ends whatever its line searches did.
+static long long iteration_cap(const wf_opts* o) {
+  const int every = o->check_every > 0 ? o->check_every : 16;
+  return ((long long)o->max_iter / every + 2) * every;
+}
+
 // Whether the graph in hand was captured with the solve's current settings.
 static bool graph_current(const wf_problem* p, const WfSolver* S, cudaStream_t st) {
   const wf_opts* o = &S->o;
   const WfScalarArgs& A = S->A;
-  const int chunk = o->check_every > 0 ? o->check_every : 16;
+  const int chunk = check_chunk(o);
   return S->exec && S->g_chunk == chunk && S->g_maxit == o->max_iter && S->g_gtol2 == A.gtol2 &&
          S->g_dchi2 == A.dchi2 && S->g_m == o->lbfgs_m && S->g_ls == A.ls && S->g_c1 == A.c1 && S->g_c2 == A.c2 &&
          S->g_inject == o->inject_timeout_map && S->g_spin == o->spin_limit && S->g_variant == variant_code(p->g) &&
          S->g_hist == A.hist && S->g_hcap == A.hcap && S->g_stream == st;
 }
 
+// Capture the iterations between two polls in a CUDA graph on st (unless the
+// graph in hand was captured with the same settings).  Every kernel's attributes
+// must have been set outside capture: one plain iteration has run before.
 template <typename T>
 static wf_status build_graph(wf_problem* p, WfSolver* S, cudaStream_t st) {
   const wf_opts* o = &S->o;
@@ -886,7 +901,7 @@ static wf_status build_graph(wf_problem* p, WfSolver* S, cudaStream_t st) {
   const WfBufs b = wf_bufs(p);
   const WfLbBufs lb = lb_bufs<T>(S);
   const int m = o->lbfgs_m;
-  const int chunk = o->check_every > 0 ? o->check_every : 16;
+  const int chunk = check_chunk(o);
   if (graph_current(p, S, st)) return WF_OK;
   if (S->exec) { cudaGraphExecDestroy(S->exec); S->exec = nullptr; }
   cudaGraph_t graph;
@@ -992,7 +1007,7 @@ static wf_status step_impl(wf_problem* p, int n_iter, int* n_active) {
   WfLbBufs lb = lb_bufs<T>(S);
   // iterations per graph launch: the graph's own count (a resumed solve
   // captures its graph below, so this is read again after the capture)
-  int chunk = S->g_chunk > 0 ? S->g_chunk : (o->check_every > 0 ? o->check_every : 16);
+  int chunk = S->g_chunk > 0 ? S->g_chunk : check_chunk(o);
   int done = 0;
   while (done < n_iter) {
     if (o->refresh_every > 0 && S->iters > 0 && S->iters % o->refresh_every == 0)
@@ -1167,11 +1182,10 @@ static wf_status refined_impl(wf_problem* p, const wf_opts* o, double tol, int m
     const WfSeed sd{(const double*)S->r_g64, res, tol};
     rs = start_impl<T>(p, &oi, nullptr, &sd);
     if (rs != WF_OK) return rs;
-    const int chunk = oi.check_every > 0 ? oi.check_every : 16;
-    const long long max_chunks = (long long)oi.max_iter / chunk + 2;
-    for (long long c = 0; c < max_chunks; ++c) {
+    const int chunk = check_chunk(&oi);
+    for (long long done = 0, cap = iteration_cap(&oi); done < cap; done += chunk) {
       int nact = 0;
-      rs = step_impl<T>(p, chunk, &nact);
+      rs = step_impl<T>(p, (int)std::min<long long>(chunk, cap - done), &nact);
       if (rs != WF_OK) return rs;
       if (nact == 0) break;
     }
@@ -1323,11 +1337,10 @@ extern "C" wf_status wf_map_solve(wf_problem* p, const wf_opts* opts, const void
   else wf_opts_default(&o);
   wf_status s = wf_solver_start(p, &o, s0);
   if (s != WF_OK) return s;
-  const int chunk = o.check_every > 0 ? o.check_every : 16;
-  const long long max_chunks = (long long)o.max_iter / chunk + 2;
-  for (long long c = 0; c < max_chunks; ++c) {
+  const int chunk = check_chunk(&o);
+  for (long long done = 0, cap = iteration_cap(&o); done < cap; done += chunk) {
     int nact = 0;
-    s = wf_solver_step(p, chunk, &nact);
+    s = wf_solver_step(p, (int)std::min<long long>(chunk, cap - done), &nact);
     if (s != WF_OK) return s;
     if (nact == 0) break;
   }
@@ -1428,7 +1441,9 @@ extern "C" wf_status wf_map_solve_many(wf_problem* const* ps, int np, const wf_o
   wf_opts o;
   if (opts) o = *opts;
   else wf_opts_default(&o);
-  const int chunk = o.check_every > 0 ? o.check_every : 16;
+  int chunk = check_chunk(&o);
+  if (chunk == o.max_iter && chunk > 1) --chunk;  // one iteration runs before the rounds
+  if (chunk < 1) chunk = 1;
   cudaStream_t us = (cudaStream_t)o.stream;
   std::vector<cudaEvent_t> ev((size_t)np + 1, nullptr);
   cudaStream_t bs = nullptr;
@@ -1523,8 +1538,7 @@ extern "C" wf_status wf_map_solve_many(wf_problem* const* ps, int np, const wf_o
   }
   std::vector<int> live((size_t)np, 1);
   std::vector<long long> last_refresh((size_t)np, 0);
-  const long long max_rounds = (long long)o.max_iter / chunk + 2;
-  for (long long r = 0; r < max_rounds && rs == WF_OK; ++r) {
+  for (long long done = 0, cap = iteration_cap(&o); done < cap && rs == WF_OK; done += chunk) {
     for (int i = 0; i < np && rs == WF_OK; ++i) {  // refreshes that are due, on the batch stream
       WfSolver* S = ps[i]->solver;
       if (o.refresh_every > 0 && live[i] && S->iters / o.refresh_every > last_refresh[i]) {

@@ -32,7 +32,7 @@
 // sequence a + i b, which carries both real transforms.
 //
 // What bounds them: HBM and instruction issue for FP32, the FP64 units for FP64
-// (two lanes an SM): so every transcendental, square root and division is taken
+// (two lanes a clock and SM): so every transcendental, square root and division is taken
 // out of the maps' passes, and the FP32 path's FP64-accurate sums run in pairs of
 // floats.  One value per thread and pass with sincospi twiddles and radices up to
 // 7 had taken, 64 maps of 768^2 FP32: 0.40 + 1.64 + 0.61 + 0.08 ms; 8 E/B maps of

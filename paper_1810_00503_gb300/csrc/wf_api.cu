@@ -120,6 +120,8 @@ WfGeo wf_make_geo(int ny, int nx, int C, int B, bool f64) {
   if (g.ncomb > g.maxblk) g.maxblk = g.ncomb;
   const int wide = wf_rg_tc(ny, C, 1, f64), tiles = (g.h + wide - 1) / wide;
   if (tiles > g.maxblk) g.maxblk = tiles;
+  const int rows = 8 * wf_rg_rows(nx, f64), blocks = (C * ny + rows - 1) / rows;
+  if (blocks > g.maxblk) g.maxblk = blocks;
   g.colinv_kind = WF_COLINV_REG_K;
   g.row_kind = WF_ROW_REG_K;
   wf_geo_tiles(g, 1, 1);

@@ -233,7 +233,7 @@ struct WfGeo {
   int maxblk;      // stride of the partial-sum slots: covers every tile choice
   int colinv_kind, row_kind;  // WF_COLINV_*_K, WF_ROW_*_K
   int tc_div, rb_div;         // TC and RB are the widest tile divided by these (1, 2, 4)
-  bool f64;                   // working type: FP64 sequences of 512 take twice the threads (wf_reg.cuh)
+  bool f64;                   // FP64 working type
   int col_plan, row_plan;     // radix plan of the TMA-fed stage's passes; row_plan is carried only (0..WF_NPLAN-1)
 };
 
@@ -244,11 +244,17 @@ WfGeo wf_make_geo(int ny, int nx, int C, int B, bool f64);
 // widest: what the objective's passes run (the L-BFGS stages are tuned).
 WfGeo wf_make_geo_pass(int ny, int nx, int C, int B, bool f64);
 
+// Lengths at which the register-resident stages split the butterflies of their
+// second pass over two threads (wf_reg.cuh).
+__host__ __device__ constexpr bool wf_rg_split(int N, bool f64, bool row) {
+  return f64 ? N == 32 || N == 128 || N == 512 : N == 512 && !row;
+}
 // Register-resident stages.  Widest tile: wf_rg_seq(N) sequences a block (256
-// threads from 64 rows up; 64-byte rows of a tile at 1024, 128-byte rows and
-// more below), and 1/2 and 1/4 of it.
+// threads from 64 rows up; 64-byte rows of a tile at 512 and 1024 in FP32, 128-byte
+// rows and more below), and 1/2 and 1/4 of it.
 __host__ __device__ constexpr int wf_rg_seq(int N, bool f64) {
-  return N == 1024 || (N == 512 && f64) ? 8 : N >= 256 ? 16 : 32;
+  const int seq = N == 1024 ? 8 : N >= 256 ? 16 : 32;
+  return wf_rg_split(N, f64, false) && N >= 128 ? seq / 2 : seq;
 }
 __host__ __device__ constexpr int wf_rg_tc(int N, int C, int div, bool f64) {
   const int seq = N == 8 && div == 4 ? 16 : wf_rg_seq(N, f64) / div;  // at least a warp a block
@@ -256,7 +262,8 @@ __host__ __device__ constexpr int wf_rg_tc(int N, int C, int div, bool f64) {
 }
 // Rows a warp of the row stage takes: pairs of rows, 32 or fewer values a thread.
 __host__ __device__ constexpr int wf_rg_rows(int nx, bool f64) {
-  return nx == 1024 || (nx == 512 && f64) ? 2 : nx >= 256 ? 4 : nx >= 64 ? 8 : nx >= 16 ? 16 : 32;
+  const int rows = nx == 1024 ? 2 : nx >= 256 ? 4 : nx >= 64 ? 8 : nx >= 16 ? 16 : 32;
+  return wf_rg_split(nx, f64, true) ? rows / 2 : rows;
 }
 // Blocks per map of the band reductions: about 4096 modes each, at most 64.
 inline int wf_band_nblk(const WfGeo& g) {

@@ -27,7 +27,7 @@
 // Measured, 120 maps of 1024^2, FP32 (bytes at 6.78 TB/s: 0.15, 0.30 and 0.22
 // ms): inverse column stage 0.466 -> 0.248 ms, row stage with data 0.533 -> 0.330
 // ms, forward column stage 0.626 -> 0.393 ms; the objective pass 1.637 -> 0.985
-// ms.  53 E/B maps of 512^2, Hessian-vector product: 0.448 -> 0.302 ms.
+// ms.  53 E/B maps of 512^2, Hessian-vector product: 0.448 -> 0.272 ms.
 #pragma once
 #include "wf_ops.cuh"
 
@@ -43,17 +43,26 @@ template <> struct WfReg<32> { static constexpr int NV = 8, RA = 4, RB = 8; };
 template <> struct WfReg<16> { static constexpr int NV = 4, RA = 4, RB = 4; };
 template <> struct WfReg<8> { static constexpr int NV = 4, RA = 2, RB = 4; };
 // Passes in the working type: R1, R2 of the column and the forward row transforms,
-// I1, I2 of the inverse row transform (the radices the other way round).  FP64 at
-// 512 holds 16 values a thread and splits the radix-32 butterflies of pass 2 over
-// two threads: a warp's FP64 instruction holds its unit for 64 cycles, so a map's
-// time is that of one warp's instructions until every unit has a warp, and 32
-// values a thread make only 128 warps of a 512^2 map.  One map of 512^2, the
-// objective pass: 186 -> 111 us.  It costs nothing where
-// the chip is full (40 maps: 1.65 -> 1.60 ms).
-template <typename T, int N> struct WfRegT {
-  static constexpr int NV = WfReg<N>::NV, R1 = WfReg<N>::RB, R2 = WfReg<N>::RA, I1 = R2, I2 = R1;
+// I1, I2 of the inverse row transform (the radices the other way round).  At the
+// lengths of wf_rg_split a thread holds half as many values and pass 2 splits its
+// butterflies, of twice as many, over two threads (wf_rg_read), for 20 operations
+// more per pair of values: twice the warps.
+//   FP64, 32, 128 and 512: a warp's FP64 instruction holds its unit for 64 cycles,
+//     so a pass over few maps takes as long as one warp's instructions.  Objective
+//     pass of one map, us: 32^2 45 -> 32, 128^2 87 -> 60, 512^2 186 -> 111; 40 maps
+//     of 512^2 1650 -> 1597.  (Where the units are busy the extra work shows: 100
+//     maps of 128^2 224 -> 257.)  8 gained nothing; 64, 256 and 1024 have no such split.
+//   FP32 columns of 512: 80 registers and three blocks an SM against 128 and two.
+//     Hessian-vector product of 53 E/B maps 302 -> 272 us, 20 E/B solves 2.42 ->
+//     2.08 ms, objective of one map 44 -> 38 us, of 256 maps 515 -> 521.
+// FP32 rows of 512 and the shorter FP32 lengths were slower split (300 maps of 32 x
+// 512: 58.6 against 70.1 us; 300 E/B maps of 128^2: 98.7 against 105.4).
+template <typename T, int N, bool ROW> struct WfRegT {
+  static constexpr bool SPLIT = wf_rg_split(N, sizeof(T) == 8, ROW);
+  static constexpr int NV = SPLIT ? WfReg<N>::NV / 2 : WfReg<N>::NV;
+  static constexpr int R1 = SPLIT ? NV : WfReg<N>::RB, R2 = SPLIT ? 2 * NV : WfReg<N>::RA;
+  static constexpr int I1 = SPLIT ? R1 : R2, I2 = SPLIT ? R2 : R1;
 };
-template <> struct WfRegT<double, 512> { static constexpr int NV = 16, R1 = 16, R2 = 32, I1 = 16, I2 = 32; };
 
 __device__ __forceinline__ float wf_fma(float a, float b, float c) { return fmaf(a, b, c); }
 __device__ __forceinline__ double wf_fma(double a, double b, double c) { return fma(a, b, c); }
@@ -234,8 +243,8 @@ template <typename T, int NV> __host__ __device__ constexpr int wf_rg_minb(int t
 // the map (h < TC) has idle columns: they load the last one and store nothing.
 // ---------------------------------------------------------------------------
 template <typename T, int C, int N, int TC> struct WfRegCol {
-  static constexpr int NV = WfRegT<T, N>::NV, G = N / NV, S = C * TC, THREADS = S * G;
-  static constexpr int R1 = WfRegT<T, N>::R1, R2 = WfRegT<T, N>::R2;
+  static constexpr int NV = WfRegT<T, N, false>::NV, G = N / NV, S = C * TC, THREADS = S * G;
+  static constexpr int R1 = WfRegT<T, N, false>::R1, R2 = WfRegT<T, N, false>::R2;
   static constexpr int PITCH = WfXch<T, S, R2>::PITCH;
   static constexpr size_t XCH = (size_t)R1 * PITCH;            // values of the exchange buffer
   static constexpr size_t SMEM = (XCH + N) * sizeof(V2<T>);    // and the twiddles
@@ -589,8 +598,8 @@ __device__ __forceinline__ void wf_rg_lb_colfwd(const WfGeo& geo, const V2<T>* P
 // values in registers, r2c from there, store.
 // ---------------------------------------------------------------------------
 template <typename T, int NX> struct WfRegRow {
-  static constexpr int NV = WfRegT<T, NX>::NV, G = NX / NV, SEQ = 32 / G;
-  static constexpr int I1 = WfRegT<T, NX>::I1, I2 = WfRegT<T, NX>::I2, F1 = WfRegT<T, NX>::R1, F2 = WfRegT<T, NX>::R2;
+  static constexpr int NV = WfRegT<T, NX, true>::NV, G = NX / NV, SEQ = 32 / G;
+  static constexpr int I1 = WfRegT<T, NX, true>::I1, I2 = WfRegT<T, NX, true>::I2, F1 = WfRegT<T, NX, true>::R1, F2 = WfRegT<T, NX, true>::R2;
   static constexpr int PI = WfXch<T, 1, I2>::PITCH, PF = WfXch<T, 1, F2>::PITCH;  // inverse, forward
   static constexpr int XI = I1 * PI, XF = F1 * PF, XM = XI > XF ? XI : XF;
   // a sequence's exchange places; the sequences of a half-warp sit G values apart

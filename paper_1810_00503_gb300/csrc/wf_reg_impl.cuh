@@ -6,7 +6,7 @@
 #include "wf_reg.cuh"
 
 template <typename T, int C, int IN, int N, int TC>
-__global__ void __launch_bounds__(WfRegCol<T, C, N, TC>::THREADS, wf_rg_minb<T, WfRegT<T, N>::NV>(WfRegCol<T, C, N, TC>::THREADS))
+__global__ void __launch_bounds__(WfRegCol<T, C, N, TC>::THREADS, wf_rg_minb<T, WfRegT<T, N, false>::NV>(WfRegCol<T, C, N, TC>::THREADS))
 k_rg_colinv(WfGeo g, const void* src_, const T* sp_, long long sp_stride, void* scratch_, const void* tw_) {
   const int b = blockIdx.y;
   const size_t st = (size_t)C * N * (IN == WF_IN_PK ? g.h : g.h + 1);
@@ -14,7 +14,7 @@ k_rg_colinv(WfGeo g, const void* src_, const T* sp_, long long sp_stride, void* 
                                 (V2<T>*)scratch_ + (size_t)b * C * N * g.h, tw_, blockIdx.x * TC);
 }
 template <typename T, int C, int IN, int N, int TC>
-__global__ void __launch_bounds__(WfRegCol<T, C, N, TC>::THREADS, wf_rg_minb<T, WfRegT<T, N>::NV>(WfRegCol<T, C, N, TC>::THREADS))
+__global__ void __launch_bounds__(WfRegCol<T, C, N, TC>::THREADS, wf_rg_minb<T, WfRegT<T, N, false>::NV>(WfRegCol<T, C, N, TC>::THREADS))
 k_rg_colfwd(WfGeo g, const void* src_, const T* sp_, long long sp_stride, const void* scratch_, void* dst_,
             double* part, const void* tw_) {
   const int b = blockIdx.y;
@@ -24,14 +24,14 @@ k_rg_colfwd(WfGeo g, const void* src_, const T* sp_, long long sp_stride, const 
                                 part + (size_t)b * WF_NSLOT * g.maxblk, tw_, blockIdx.x * TC, blockIdx.x);
 }
 template <typename T, int C, int N, int TC>
-__global__ void __launch_bounds__(WfRegCol<T, C, N, TC>::THREADS, wf_rg_minb<T, WfRegT<T, N>::NV>(WfRegCol<T, C, N, TC>::THREADS))
+__global__ void __launch_bounds__(WfRegCol<T, C, N, TC>::THREADS, wf_rg_minb<T, WfRegT<T, N, false>::NV>(WfRegCol<T, C, N, TC>::THREADS))
 k_rg_colsim(WfGeo g, const T* sp_, long long sp_stride, void* scratch_, const void* tw_) {
   const int b = blockIdx.y;
   wf_rg_colsim<T, C, N, TC>(g, sp_ + (size_t)b * sp_stride, (V2<T>*)scratch_ + (size_t)b * C * N * g.h, tw_,
                             blockIdx.x * TC);
 }
 template <typename T, int MODE, int NX>
-__global__ void __launch_bounds__(256, wf_rg_minb<T, WfRegT<T, NX>::NV>(256))
+__global__ void __launch_bounds__(256, wf_rg_minb<T, WfRegT<T, NX, true>::NV>(256))
 k_rg_row(WfGeo g, void* scratch_, const void* d_, const void* w_, const void* aux_, void* out_, double* part,
          const void* tw_) {
   wf_rg_row<T, MODE, NX>(g, (V2<T>*)scratch_, (const T*)d_, (const T*)w_, (const T*)aux_, (T*)out_, part, tw_,
@@ -41,17 +41,17 @@ k_rg_row(WfGeo g, void* scratch_, const void* d_, const void* w_, const void* au
 // The same stages on the direction P[next] of every map still iterating (device
 // functions in wf_reg.cuh, shared with the launches over several problems).
 template <typename T, int C, int N, int TC>
-__global__ void __launch_bounds__(WfRegCol<T, C, N, TC>::THREADS, wf_rg_minb<T, WfRegT<T, N>::NV>(WfRegCol<T, C, N, TC>::THREADS))
+__global__ void __launch_bounds__(WfRegCol<T, C, N, TC>::THREADS, wf_rg_minb<T, WfRegT<T, N, false>::NV>(WfRegCol<T, C, N, TC>::THREADS))
 k_rg_lb_colinv(WfGeo g, WfBufs b, WfLbBufs lb) {
   wf_rg_lb_colinv_map<T, C, N, TC>(g, b, lb, blockIdx.y, blockIdx.x);
 }
 template <typename T, int NX>
-__global__ void __launch_bounds__(256, wf_rg_minb<T, WfRegT<T, NX>::NV>(256))
+__global__ void __launch_bounds__(256, wf_rg_minb<T, WfRegT<T, NX, true>::NV>(256))
 k_rg_lb_row(WfGeo g, WfBufs b, WfLbBufs lb) {
   wf_rg_lb_row_map<T, NX>(g, b, lb, blockIdx.y, blockIdx.x);
 }
 template <typename T, int C, int N, int TC>
-__global__ void __launch_bounds__(WfRegCol<T, C, N, TC>::THREADS, wf_rg_minb<T, WfRegT<T, N>::NV>(WfRegCol<T, C, N, TC>::THREADS))
+__global__ void __launch_bounds__(WfRegCol<T, C, N, TC>::THREADS, wf_rg_minb<T, WfRegT<T, N, false>::NV>(WfRegCol<T, C, N, TC>::THREADS))
 k_rg_lb_colfwd(WfGeo g, WfBufs b, WfLbBufs lb) {
   wf_rg_lb_colfwd_map<T, C, N, TC>(g, b, lb, blockIdx.y, blockIdx.x);
 }

@@ -394,8 +394,8 @@ def run_eval_any(dev, hbm, B=64, ny=768, nx=768, reps=10):
     achieved = alg / (ms / 1000.0) / 1e9
     return {"evals_per_s": B * 1000.0 / ms, "ms_per_call": ms, "maps": B, "shape": [ny, nx],
             "algorithmic_bytes_per_call": alg, "achieved_GBps": achieved, "frac": achieved / hbm,
-            "note": "wf_eval_any, mixed precision, radix 4 x 4 x 4 x 4 x 3 transforms; per call including its "
-                    "scratch allocation, free and synchronisation"}
+            "note": "wf_eval_any, mixed precision, mixed-radix transforms; per call including its "
+                    "scratch and synchronisation"}
 
 
 def run_hetero(args, dev, count=256, n_bands=10, sizes=(64, 128, 256, 512, 1024)):
@@ -455,7 +455,7 @@ def run_hetero(args, dev, count=256, n_bands=10, sizes=(64, 128, 256, 512, 1024)
             "evals_per_s": evals / dt, "stop": "||g||/||g0|| < 1e-6", "statuses": statuses,
             "dchi2_dlogq": {"bands": n_bands, "ms_per_batch": dq_dt * 1e3, "maps_per_s": count / dq_dt},
             "note": "one problem per size, all sizes solved as one batch by wf_map_solve_many: each iteration "
-                    "is seven launches shared by the five sizes (ping-pong stages, tile widths tuned per size), each "
+                    "is seven launches shared by the five sizes (register-resident stages, tile widths tuned per size), each "
                     "round of 32 iterations one graph launch; a 2-iteration solve first tunes and sets up the solvers"}
 
 
@@ -600,7 +600,7 @@ def iteration_flops(n, m):
     overcounts the radix-8/16 butterflies.  Returns (flops, source)."""
     import math
     if (n, m) in FP64_ITERATION_FLOPS_COUNTED:
-        return FP64_ITERATION_FLOPS_COUNTED[(n, m)], "ncu FP64 instruction counters"
+        return FP64_ITERATION_FLOPS_COUNTED[(n, m)], "ncu FP64 instruction counters of the three-pass stages"
     h = n // 2
     fft = 5 * (h * n * math.log2(n) + n * h * math.log2(h))
     vals = n * h

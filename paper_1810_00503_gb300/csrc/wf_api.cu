@@ -1,5 +1,6 @@
 // C ABI of the Wiener-filter library: handle, prepared problems and the
 // single-pass operator calls.  The L-BFGS driver lives in wf_solve.cu.
+#include <algorithm>
 #include <math.h>
 #include <stdarg.h>
 #include <stdio.h>
@@ -433,7 +434,9 @@ extern "C" wf_status wf_problem_create_rect(wf_handle* h, const wf_map* maps, in
   if (s == WF_OK) s = wf_alloc(h, &p->w, npix * count * p->elt, "weights");
   if (s == WF_OK) s = wf_alloc(h, &p->sp, nsp * (shared ? 1 : count) * p->elt, "sqrt(P) tables");
   if (s == WF_OK) s = wf_alloc(h, &p->scratch, npix * count * p->elt, "scratch");
-  if (s == WF_OK) s = wf_alloc(h, (void**)&p->part, sizeof(double) * WF_NSLOT * p->g.maxblk * count, "partial sums");
+  // the stride of either working type: a MIXED problem's refined solve evaluates in FP64
+  const int maxblk = std::max(p->g.maxblk, wf_make_geo(ny, nx, C, count, true).maxblk);
+  if (s == WF_OK) s = wf_alloc(h, (void**)&p->part, sizeof(double) * WF_NSLOT * maxblk * count, "partial sums");
   if (s == WF_OK) s = wf_alloc(h, (void**)&p->flags, sizeof(int) * 4, "flags");
   if (s != WF_OK) { free_problem(p); return s; }
   cudaStream_t st = (cudaStream_t)stream;

@@ -1131,8 +1131,9 @@ static wf_status refined_impl(wf_problem* p, const wf_opts* o, double tol, int m
   WF_TRY(cudaStreamWaitEvent(st, S->ev_in, 0));
   // The FP64 operator of the outer evaluations: for a MIXED problem on exact
   // FP64 copies of the working-precision inputs (the problem the inner solves
-  // see), always on the default tiles.
-  const WfGeo& go = p->gp;
+  // see).  Its tiles are the FP64 stages' own: the problem's (p->gp) are those of
+  // the working type, which differ at sides of 32, 128 and 512.
+  const WfGeo go = wf_make_geo_pass(p->n, p->nx, p->C, B, true);
   WfBufs bo = wf_bufs(p);
   if (mixed) {
     k_convert<float, double><<<wf_grid(per * B), 256, 0, st>>>((const float*)p->d, (double*)S->r_d64, per * B);

@@ -10,6 +10,17 @@
 #include "wf_multi.cuh"
 #include "wf_reg.cuh"
 
+// f(N) of every length.
+template <class F> constexpr void wf_multi_lengths(F& f) {
+  f(std::integral_constant<int, 8>());
+  f(std::integral_constant<int, 16>());
+  f(std::integral_constant<int, 32>());
+  f(std::integral_constant<int, 64>());
+  f(std::integral_constant<int, 128>());
+  f(std::integral_constant<int, 256>());
+  f(std::integral_constant<int, 512>());
+  f(std::integral_constant<int, 1024>());
+}
 // f<N>() of length n.
 template <class F> __device__ __forceinline__ void wf_rg_switch(int n, F&& f) {
   switch (n) {
@@ -73,6 +84,31 @@ template <typename T> inline size_t wf_multi_row_smem(const WfGeo& g) {
   return sm;
 }
 
+// The most shared memory a stage of any problem asks for: the widest column tiles
+// of C channels, and row blocks of eight warps.  Neither is the length 1024's
+// everywhere: FP32 rows of 512 have the largest row block.
+template <typename T, int C> constexpr size_t wf_multi_col_max() {
+  size_t m = 0;
+  auto take = [&](auto n) {
+    constexpr int N = decltype(n)::value;
+    constexpr size_t s = WfRegCol<T, C, N, wf_rg_tc(N, C, 1, sizeof(T) == 8)>::SMEM;
+    constexpr size_t t = WfRegCol<T, C, N, wf_rg_tc(N, C, 2, sizeof(T) == 8)>::SMEM;
+    m = s > m ? s : m;
+    m = t > m ? t : m;
+  };
+  wf_multi_lengths(take);
+  return m;
+}
+template <typename T> constexpr size_t wf_multi_row_max() {
+  size_t m = 0;
+  auto take = [&](auto n) {
+    constexpr size_t s = WfRegRow<T, decltype(n)::value>::smem(8);
+    m = s > m ? s : m;
+  };
+  wf_multi_lengths(take);
+  return m;
+}
+
 template <typename T, int C>
 cudaError_t wf_launch_multi_fft(const WfMultiArgs& a, int stage, cudaStream_t st) {
   static int done[3] = {0, 0, 0};
@@ -84,7 +120,8 @@ cudaError_t wf_launch_multi_fft(const WfMultiArgs& a, int stage, cudaStream_t st
     if (s > sm) sm = s;
   }
   auto k = row ? k_multi_row<T> : stage == 0 ? k_multi_col<T, C, true> : k_multi_col<T, C, false>;
-  cudaError_t e = wfimpl::ensure_smem(k, WfRegCol<T, 1, 1024, wf_rg_tc(1024, 1, 1, sizeof(T) == 8)>::SMEM, &done[stage]);  // the largest
+  constexpr size_t most_col = wf_multi_col_max<T, C>(), most_row = wf_multi_row_max<T>();
+  cudaError_t e = wfimpl::ensure_smem(k, row ? most_row : most_col, &done[stage]);
   if (e != cudaSuccess) return e;
   k<<<r.start[a.np], 256, sm, st>>>(r, a);
   return cudaGetLastError();

@@ -17,7 +17,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 OBJ = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libwf.so")
-SOURCES = ["wf_api.cu", "wf_solve.cu", "wf_ops_f32.cu", "wf_ops_f64.cu", "wf_lbcol_f32.cu", "wf_lbcol_f64.cu",
+SOURCES = ["wf_api.cu", "wf_mem.cu", "wf_solve.cu", "wf_ops_f32.cu", "wf_ops_f64.cu", "wf_lbcol_f32.cu", "wf_lbcol_f64.cu",
            "wf_lbrow_f32.cu", "wf_lbrow_f64.cu", "wf_noalloc.cu", "wf_bandpower.cu", "wf_rng.cu", "wf_peak.cu",
            "wf_multi.cu", "wf_any.cu",
            "wf_multi_f32_c1.cu", "wf_multi_f32_c2.cu", "wf_multi_f64_c1.cu", "wf_multi_f64_c2.cu",

@@ -706,8 +706,13 @@ extern "C" wf_status wf_eval_any(wf_handle* h, int B, int C, int ny, int nx, int
     if (e == cudaSuccess) e = es;
     if (e != cudaSuccess) rs = wf_cuda_fail(e, "wf_eval_any");
   }
-  wf_free_idle(h, work);
-  wf_free_idle(h, scr);
+  if (rs == WF_OK) {
+    wf_free_idle(h, work);
+    wf_free_idle(h, scr);
+  } else {
+    void* ptrs[] = {work, scr};
+    wf_free_all(h, ptrs, 2);
+  }
   return rs;
 }
 

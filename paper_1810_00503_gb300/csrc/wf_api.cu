@@ -203,33 +203,6 @@ static void wf_make_twiddles_all(double2* out) {
   }
 }
 
-// The handle's memory pool; without one (no pool support) it allocates plainly.
-static void pool_create(wf_handle* h) {
-  cudaMemPoolProps pr;
-  memset(&pr, 0, sizeof pr);
-  pr.allocType = cudaMemAllocationTypePinned;
-  pr.location.type = cudaMemLocationTypeDevice;
-  pr.location.id = h->device;
-  if (cudaStreamCreateWithFlags(&h->pool_stream, cudaStreamNonBlocking) != cudaSuccess) {
-    h->pool_stream = nullptr;
-  } else if (cudaMemPoolCreate(&h->pool, &pr) != cudaSuccess) {
-    h->pool = nullptr;
-  } else {
-    unsigned long long keep = h->limit ? 0 : WF_POOL_KEEP;
-    cudaMemPoolSetAttribute(h->pool, cudaMemPoolAttrReleaseThreshold, &keep);
-  }
-  cudaGetLastError();
-}
-// Which allocations come from it.  Larger ones gain nothing that matters beside the
-// work they are for, and take 3 ms more to map for a history ring of 10 GB.
-static bool pooled(const wf_handle* h, size_t bytes) { return h->pool && bytes <= WF_POOL_ONE; }
-static void pool_destroy(wf_handle* h) {
-  if (h->pool_stream) cudaStreamSynchronize(h->pool_stream);
-  if (h->pool) cudaMemPoolDestroy(h->pool);
-  if (h->pool_stream) cudaStreamDestroy(h->pool_stream);
-  for (auto& q : h->pinned) cudaFreeHost(q.first);
-}
-
 extern "C" wf_status wf_create(wf_handle** out, size_t workspace_limit) {
   if (!out) return wf_fail(WF_EINVAL, "wf_create: null output pointer");
   *out = nullptr;
@@ -237,17 +210,15 @@ extern "C" wf_status wf_create(wf_handle** out, size_t workspace_limit) {
   if (!h) return wf_fail(WF_ENOMEM, "wf_create: host allocation failed");
   h->limit = workspace_limit;
   h->used = 0;
-  h->pool = nullptr;
-  h->pool_stream = nullptr;
   cudaError_t e = cudaGetDevice(&h->device);
   if (e != cudaSuccess) { delete h; return wf_cuda_fail(e, "wf_create: cudaGetDevice"); }
-  pool_create(h);
+  wf_mem_open(h);
   double2* tw64 = (double2*)malloc(sizeof(double2) * WF_TWTAB_ALL);
   float2* tw32 = (float2*)malloc(sizeof(float2) * WF_TWTAB_ALL);
   if (!tw64 || !tw32) {
     free(tw64);
     free(tw32);
-    pool_destroy(h);
+    wf_mem_close(h);
     delete h;
     return wf_fail(WF_ENOMEM, "wf_create: host allocation failed");
   }
@@ -268,7 +239,7 @@ extern "C" wf_status wf_create(wf_handle** out, size_t workspace_limit) {
   if (s != WF_OK || e != cudaSuccess) {
     wf_free(h, h->tw64);
     wf_free(h, h->tw32);
-    pool_destroy(h);
+    wf_mem_close(h);
     delete h;
     return s != WF_OK ? s : wf_cuda_fail(e, "wf_create: twiddle tables");
   }
@@ -280,7 +251,7 @@ extern "C" wf_status wf_destroy(wf_handle* h) {
   if (!h) return WF_OK;
   wf_free(h, h->tw64);
   wf_free(h, h->tw32);
-  pool_destroy(h);
+  wf_mem_close(h);
   delete h;
   return WF_OK;
 }
@@ -294,95 +265,10 @@ extern "C" wf_status wf_workspace_used(const wf_handle* h, size_t* bytes) {
 
 static void free_problem(wf_problem* p) {
   if (!p) return;
-  cudaDeviceSynchronize();
   void* ptrs[] = {p->d, p->w, p->sp, p->sp0, p->scratch, p->part, p->flags, p->bpart};
-  for (void* q : ptrs) wf_free_idle(p->h, q);
+  wf_free_all(p->h, ptrs, (int)(sizeof ptrs / sizeof ptrs[0]));
   wf_solver_free(p);
   free(p);
-}
-
-wf_status wf_alloc(wf_handle* h, void** ptr, size_t bytes, const char* what) {
-  *ptr = nullptr;
-  {
-    std::lock_guard<std::mutex> lock(h->mu);
-    if (h->limit && h->used + bytes > h->limit)
-      return wf_fail(WF_ENOMEM, "%s: %zu more bytes would exceed the workspace limit (%zu of %zu in use)", what,
-                     bytes, h->used, h->limit);
-    h->used += bytes;  // reserved before the allocation, so concurrent callers cannot overshoot
-  }
-  cudaError_t e;
-  if (pooled(h, bytes)) {
-    e = cudaMallocFromPoolAsync(ptr, bytes, h->pool, h->pool_stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(h->pool_stream);  // usable on every stream from here
-    if (e == cudaErrorMemoryAllocation) {  // once more without what the pool keeps
-      cudaGetLastError();
-      cudaMemPoolTrimTo(h->pool, 0);
-      e = cudaMallocFromPoolAsync(ptr, bytes, h->pool, h->pool_stream);
-      if (e == cudaSuccess) e = cudaStreamSynchronize(h->pool_stream);
-    }
-  } else {
-    e = cudaMalloc(ptr, bytes);
-  }
-  if (e != cudaSuccess) {
-    *ptr = nullptr;
-    cudaGetLastError();
-    std::lock_guard<std::mutex> lock(h->mu);
-    h->used -= bytes;
-    return wf_fail(e == cudaErrorMemoryAllocation ? WF_ENOMEM : WF_ECUDA,
-                   "device allocation of %zu bytes for %s failed: %s", bytes, what,
-                   cudaGetErrorString(e));
-  }
-  std::lock_guard<std::mutex> lock(h->mu);
-  h->live[*ptr] = bytes;
-  return WF_OK;
-}
-
-void wf_free(wf_handle* h, void* ptr) {
-  if (!ptr) return;
-  cudaDeviceSynchronize();
-  wf_free_idle(h, ptr);
-}
-
-void wf_free_idle(wf_handle* h, void* ptr) {
-  if (!ptr) return;
-  size_t bytes = 0;
-  {
-    std::lock_guard<std::mutex> lock(h->mu);
-    auto it = h->live.find(ptr);
-    if (it != h->live.end()) {
-      bytes = it->second;
-      h->live.erase(it);
-    }
-  }
-  if (pooled(h, bytes)) cudaFreeAsync(ptr, h->pool_stream);
-  else cudaFree(ptr);
-  std::lock_guard<std::mutex> lock(h->mu);
-  h->used -= bytes;
-}
-
-cudaError_t wf_pinned_alloc(wf_handle* h, void** ptr, size_t bytes) {
-  {
-    std::lock_guard<std::mutex> lock(h->mu);
-    for (size_t i = 0; i < h->pinned.size(); ++i)
-      if (h->pinned[i].second == bytes) {
-        *ptr = h->pinned[i].first;
-        h->pinned.erase(h->pinned.begin() + i);
-        return cudaSuccess;
-      }
-  }
-  return cudaMallocHost(ptr, bytes);
-}
-
-void wf_pinned_free(wf_handle* h, void* ptr, size_t bytes) {
-  if (!ptr) return;
-  {
-    std::lock_guard<std::mutex> lock(h->mu);
-    if (h->pinned.size() < WF_PINNED_KEEP) {
-      h->pinned.emplace_back(ptr, bytes);
-      return;
-    }
-  }
-  cudaFreeHost(ptr);
 }
 
 extern "C" wf_status wf_problem_create_rect(wf_handle* h, const wf_map* maps, int count, int ny, int nx, int C,
@@ -483,10 +369,7 @@ extern "C" wf_status wf_problem_create(wf_handle* h, const wf_map* maps, int cou
 }
 
 extern "C" wf_status wf_problem_destroy(wf_problem* p) {
-  if (p) {
-    cudaDeviceSynchronize();
-    free_problem(p);
-  }
+  free_problem(p);
   return WF_OK;
 }
 
@@ -551,8 +434,7 @@ static wf_status band_partials(wf_problem* p, int nb) {
   const size_t need = (size_t)p->count * wf_band_nblk(p->g) * nb;
   if (p->bpart && p->bpart_n >= need) return WF_OK;
   if (p->bpart) {
-    cudaDeviceSynchronize();  // a pending band sum may still read the old buffer
-    wf_free(p->h, p->bpart);
+    wf_free(p->h, p->bpart);  // waits: a pending band sum may still read the old buffer
     p->bpart = nullptr;
     p->bpart_n = 0;
   }

@@ -255,8 +255,7 @@ struct Scope {  // frees what the estimator allocates, on every return path
   void addp(wf_problem* p) { probs[np++] = p; }
   ~Scope() {
     for (int i = 0; i < np; ++i) wf_problem_destroy(probs[i]);
-    cudaDeviceSynchronize();
-    for (int i = 0; i < n; ++i) wf_free_idle(h, ptrs[i]);
+    wf_free_all(h, ptrs, n);
   }
 };
 }  // namespace

@@ -570,11 +570,10 @@ void wf_solver_free(wf_problem* p) {
   if (S->exec) cudaGraphExecDestroy(S->exec);
   void* ptrs[] = {S->s, S->g, S->ring, S->st, S->nact, S->stats_dev, S->hist, S->r_s64, S->r_g64, S->r_d64,
                   S->r_w64, S->r_sp64, S->r_scr64, S->r_res};
-  cudaDeviceSynchronize();
-  for (void* q : ptrs) wf_free_idle(p->h, q);
+  const bool idle = wf_free_all(p->h, ptrs, (int)(sizeof ptrs / sizeof ptrs[0]));
   if (S->r_res_host) cudaFreeHost(S->r_res_host);
-  wf_pinned_free(p->h, S->nact_host, sizeof(int));
-  wf_pinned_free(p->h, S->stats_host, sizeof(double) * 5 * S->B);
+  wf_pinned_free(p->h, S->nact_host, sizeof(int), idle);
+  wf_pinned_free(p->h, S->stats_host, sizeof(double) * 5 * S->B, idle);
   if (S->stream) cudaStreamDestroy(S->stream);
   if (S->ev_in) cudaEventDestroy(S->ev_in);
   if (S->ev_out) cudaEventDestroy(S->ev_out);

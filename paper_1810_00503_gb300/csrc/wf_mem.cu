@@ -30,8 +30,12 @@ void wf_mem_close(wf_handle* h) {
 }
 
 // Which allocations come from the pool.  Larger ones gain nothing that matters beside
-// the work they are for, and take 3 ms more to map for a history ring of 10 GB.
-static bool pooled(const wf_handle* h, size_t bytes) { return h->pool && bytes <= WF_POOL_ONE; }
+// the work they are for, and take 3 ms more to map for a history ring of 10 GB; with
+// another device current than the handle's, the memory has to be that device's.
+static bool pooled(const wf_handle* h, size_t bytes) {
+  int dev = -1;
+  return h->pool && bytes <= WF_POOL_ONE && cudaGetDevice(&dev) == cudaSuccess && dev == h->device;
+}
 
 wf_status wf_alloc(wf_handle* h, void** ptr, size_t bytes, const char* what) {
   *ptr = nullptr;
@@ -42,8 +46,9 @@ wf_status wf_alloc(wf_handle* h, void** ptr, size_t bytes, const char* what) {
                      bytes, h->used, h->limit);
     h->used += bytes;  // reserved before the allocation, so concurrent callers cannot overshoot
   }
+  const bool pool = pooled(h, bytes);
   cudaError_t e;
-  if (pooled(h, bytes)) {
+  if (pool) {
     e = cudaMallocFromPoolAsync(ptr, bytes, h->pool, h->pool_stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->pool_stream);  // usable on every stream from here
     if (e == cudaErrorMemoryAllocation) {  // once more without what the pool keeps
@@ -65,7 +70,7 @@ wf_status wf_alloc(wf_handle* h, void** ptr, size_t bytes, const char* what) {
                    cudaGetErrorString(e));
   }
   std::lock_guard<std::mutex> lock(h->mu);
-  h->live[*ptr] = bytes;
+  h->live[*ptr] = {bytes, pool};
   return WF_OK;
 }
 
@@ -88,19 +93,19 @@ static bool wait_idle(wf_handle* h) {
 // cudaFree waits by itself.
 static void release(wf_handle* h, void* ptr, bool idle) {
   if (!ptr) return;
-  size_t bytes = 0;
+  wf_handle::Block b = {0, false};
   {
     std::lock_guard<std::mutex> lock(h->mu);
     auto it = h->live.find(ptr);
     if (it != h->live.end()) {
-      bytes = it->second;
+      b = it->second;
       h->live.erase(it);
     }
   }
-  if (!pooled(h, bytes)) cudaFree(ptr);
+  if (!b.pooled) cudaFree(ptr);
   else if (idle) cudaFreeAsync(ptr, h->pool_stream);
   std::lock_guard<std::mutex> lock(h->mu);
-  h->used -= bytes;
+  h->used -= b.bytes;
 }
 
 bool wf_free_all(wf_handle* h, void* const* ptrs, int n) {

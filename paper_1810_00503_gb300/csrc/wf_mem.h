@@ -17,10 +17,12 @@ struct wf_handle {
   void* tw32;   // WF_TWTAB_ALL float2 twiddles
   size_t limit;  // workspace limit in bytes (0 = none)
   size_t used;   // device bytes held by this handle's allocations
-  // Memory pool of the handle's allocations up to WF_POOL_ONE bytes, so that a call
-  // that allocates its work space (wf_eval_any, the band powers, a problem) does not
-  // map and unmap device memory each time: 64 maps of 768^2 1.03 -> 0.73 ms a
-  // wf_eval_any call, a band-power estimate of 39 E/B maps of 256^2 4.87 -> 3.36 ms.
+  // Memory pool of the handle's allocations up to WF_POOL_ONE bytes made while its
+  // device is current (wf_eval_any runs on the current one, whatever the handle's),
+  // so that a call that allocates its work space (wf_eval_any, the band powers, a
+  // problem) does not map and unmap device memory each time: 64 maps of 768^2 1.03 ->
+  // 0.73 ms a wf_eval_any call, a band-power estimate of 39 E/B maps of 256^2 4.87 ->
+  // 3.36 ms.
   // At most WF_POOL_KEEP freed bytes stay in it (none with a workspace limit), until
   // wf_destroy or an allocation that fails without them.
   // Allocations and frees are ordered on a stream of the pool's own, and a buffer is
@@ -30,7 +32,11 @@ struct wf_handle {
   cudaStream_t pool_stream;
   std::vector<std::pair<void*, size_t>> pinned;  // freed pinned host buffers, at most WF_PINNED_KEEP
   std::mutex mu;
-  std::unordered_map<void*, size_t> live;  // allocation -> bytes
+  struct Block {
+    size_t bytes;
+    bool pooled;
+  };
+  std::unordered_map<void*, Block> live;  // the handle's allocations
   std::unordered_map<long long, int> tuned;  // (ny, nx, C, precision, maps) -> FFT-stage variant
 };
 
@@ -44,8 +50,8 @@ wf_status wf_cuda_fail(cudaError_t e, const char* what);
 // Pool of a handle whose device and limit are set, and its end.
 void wf_mem_open(wf_handle* h);
 void wf_mem_close(wf_handle* h);
-// Device allocation charged to the handle's workspace (WF_ENOMEM beyond its
-// limit), and its release; null pointers are skipped.  wf_free and wf_free_all
+// Allocation on the current device, charged to the handle's workspace (WF_ENOMEM
+// beyond its limit), and its release; null pointers are skipped.  wf_free and wf_free_all
 // first wait for the handle's device, whichever device is current, and wf_free_all
 // says whether that wait succeeded; wf_free_idle is for buffers whose last use the
 // caller has already waited for.

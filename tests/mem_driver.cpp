@@ -149,10 +149,30 @@ static int failed_wait() {
   return 0;
 }
 
+// Memory asked for while another device is current is that device's.
+static int current_device() {
+  wf_handle h;
+  open(&h, 0);
+  void *a, *b;
+  CHECK(wf_alloc(&h, &a, 1 << 20, "a") == WF_OK && g_live.at(a).dev == 0 && g_live.at(a).pool);
+  g_cur = 1;
+  CHECK(wf_alloc(&h, &b, 1 << 20, "b") == WF_OK && g_live.at(b).dev == 1);
+  g_busy[0] = g_busy[1] = true;
+  g_cur = 0;
+  wf_free(&h, b);
+  g_busy[0] = true;
+  g_cur = 1;
+  wf_free(&h, a);
+  CHECK(!g_violations && !g_busy[0] && !g_busy[1] && h.used == 0 && g_live.empty());
+  wf_mem_close(&h);
+  return 0;
+}
+
 int main(int argc, char** argv) {
   const std::string t = argc > 1 ? argv[1] : "";
   if (t == "other_device") return other_device();
   if (t == "failed_wait") return failed_wait();
+  if (t == "current_device") return current_device();
   printf("unknown test\n");
   return 2;
 }

@@ -168,7 +168,9 @@ wf_status wf_destroy(wf_handle* h);
 wf_status wf_problem_variant(const wf_problem* p, int* variant);
 
 /* Device bytes the handle holds now (twiddle tables, problems, solver state).
- * Plumbing. */
+ * A handle without a workspace limit keeps up to 1 GB of freed buffers of 256 MB
+ * or less for its next calls, not counted here; wf_destroy gives them back, and so
+ * does an allocation of any handle that fails without them.  Plumbing. */
 wf_status wf_workspace_used(const wf_handle* h, size_t* bytes);
 
 /* Message for the last failing call on this thread ("" if none).  The pointer

@@ -2,7 +2,14 @@
 // wait before a buffer is given back.
 #include <string.h>
 
+#include <algorithm>
+
 #include "wf_mem.h"
+
+// Handles whose pools may hold freed memory; never destroyed, as a handle may be
+// closed while the process ends.
+static std::mutex g_open_mu;
+static std::vector<wf_handle*>& g_open = *new std::vector<wf_handle*>();
 
 // Without pool support the handle allocates plainly.
 void wf_mem_open(wf_handle* h) {
@@ -21,8 +28,14 @@ void wf_mem_open(wf_handle* h) {
     cudaMemPoolSetAttribute(h->pool, cudaMemPoolAttrReleaseThreshold, &keep);
   }
   cudaGetLastError();
+  std::lock_guard<std::mutex> lock(g_open_mu);
+  g_open.push_back(h);
 }
 void wf_mem_close(wf_handle* h) {
+  {
+    std::lock_guard<std::mutex> lock(g_open_mu);
+    g_open.erase(std::remove(g_open.begin(), g_open.end(), h), g_open.end());
+  }
   if (h->pool_stream) cudaStreamSynchronize(h->pool_stream);
   if (h->pool) cudaMemPoolDestroy(h->pool);
   if (h->pool_stream) cudaStreamDestroy(h->pool_stream);
@@ -37,6 +50,23 @@ static bool pooled(const wf_handle* h, size_t bytes) {
   return h->pool && bytes <= WF_POOL_ONE && cudaGetDevice(&dev) == cudaSuccess && dev == h->device;
 }
 
+// Give back what the pools of every handle of device dev keep.
+static void trim_pools(int dev) {
+  std::lock_guard<std::mutex> lock(g_open_mu);
+  for (wf_handle* h : g_open)
+    if (h->pool && h->device == dev) {
+      cudaStreamSynchronize(h->pool_stream);  // frees still on their way are given back too
+      cudaMemPoolTrimTo(h->pool, 0);
+    }
+}
+
+// One attempt at an allocation on the current device.
+static cudaError_t allocate(wf_handle* h, void** ptr, size_t bytes, bool pool) {
+  if (!pool) return cudaMalloc(ptr, bytes);
+  const cudaError_t e = cudaMallocFromPoolAsync(ptr, bytes, h->pool, h->pool_stream);
+  return e == cudaSuccess ? cudaStreamSynchronize(h->pool_stream) : e;  // usable on every stream from here
+}
+
 wf_status wf_alloc(wf_handle* h, void** ptr, size_t bytes, const char* what) {
   *ptr = nullptr;
   {
@@ -47,18 +77,12 @@ wf_status wf_alloc(wf_handle* h, void** ptr, size_t bytes, const char* what) {
     h->used += bytes;  // reserved before the allocation, so concurrent callers cannot overshoot
   }
   const bool pool = pooled(h, bytes);
-  cudaError_t e;
-  if (pool) {
-    e = cudaMallocFromPoolAsync(ptr, bytes, h->pool, h->pool_stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(h->pool_stream);  // usable on every stream from here
-    if (e == cudaErrorMemoryAllocation) {  // once more without what the pool keeps
-      cudaGetLastError();
-      cudaMemPoolTrimTo(h->pool, 0);
-      e = cudaMallocFromPoolAsync(ptr, bytes, h->pool, h->pool_stream);
-      if (e == cudaSuccess) e = cudaStreamSynchronize(h->pool_stream);
-    }
-  } else {
-    e = cudaMalloc(ptr, bytes);
+  cudaError_t e = allocate(h, ptr, bytes, pool);
+  int dev = 0;
+  if (e == cudaErrorMemoryAllocation && cudaGetDevice(&dev) == cudaSuccess) {  // once more without what the pools keep
+    cudaGetLastError();
+    trim_pools(dev);
+    e = allocate(h, ptr, bytes, pool);
   }
   if (e != cudaSuccess) {
     *ptr = nullptr;

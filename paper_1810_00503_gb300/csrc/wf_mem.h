@@ -24,7 +24,9 @@ struct wf_handle {
   // 0.73 ms a wf_eval_any call, a band-power estimate of 39 E/B maps of 256^2 4.87 ->
   // 3.36 ms.
   // At most WF_POOL_KEEP freed bytes stay in it (none with a workspace limit), until
-  // wf_destroy or an allocation that fails without them.
+  // wf_destroy or until an allocation of any handle, from a pool or not, fails
+  // without them.  They are not in `used`, and other allocators of the process
+  // cannot reach them.
   // Allocations and frees are ordered on a stream of the pool's own, and a buffer is
   // freed only when nothing uses it any more, so any stream and thread may use the
   // handle's buffers as before.  nullptr: plain cudaMalloc.

@@ -168,11 +168,49 @@ static int current_device() {
   return 0;
 }
 
+// What the pools keep is given back when an allocation fails without it: one from a
+// pool, one too large for a pool, and one of another handle; one that does not fit
+// all the same stays refused and uncharged.
+static int trims() {
+  const size_t one = WF_POOL_ONE, most = 4 * one;
+  g_room[0] = most;
+  wf_handle h, k;
+  open(&h, 0);
+  open(&k, 0);
+  for (int round = 0; round < 3; ++round) {
+    void *a[3], *b;
+    for (void*& p : a) CHECK(wf_alloc(&h, &p, one, "a") == WF_OK);
+    CHECK(wf_free_all(&h, a, 3) && g_room[0] == one);
+    wf_handle* who = round == 2 ? &k : &h;
+    if (round == 0) {  // from the pool, while a buffer of 3 is in use elsewhere
+      g_room[0] = 0;
+      ((Pool*)h.pool)->kept = one / 2;
+      ((Pool*)k.pool)->kept = one / 2;
+      CHECK(wf_alloc(&h, &b, one, "b") == WF_OK);
+      wf_free(&h, b);
+      g_room[0] = one;
+      ((Pool*)h.pool)->kept = 3 * one;
+      ((Pool*)k.pool)->kept = 0;
+    }
+    CHECK(wf_alloc(who, &b, 2 * one, "b") == WF_OK);
+    const size_t used = who->used;
+    void* c;
+    CHECK(wf_alloc(who, &c, 3 * one, "c") == WF_ENOMEM && !c && who->used == used);
+    wf_free(who, b);
+    CHECK(who->used == 0);
+  }
+  wf_mem_close(&k);
+  wf_mem_close(&h);
+  CHECK(g_room[0] == most && g_live.empty());
+  return 0;
+}
+
 int main(int argc, char** argv) {
   const std::string t = argc > 1 ? argv[1] : "";
   if (t == "other_device") return other_device();
   if (t == "failed_wait") return failed_wait();
   if (t == "current_device") return current_device();
+  if (t == "trims") return trims();
   printf("unknown test\n");
   return 2;
 }

@@ -33,8 +33,8 @@
 //
 // What bounds them: HBM and instruction issue for FP32, the FP64 units for FP64
 // (two lanes a clock and SM): so every transcendental, square root and division is taken
-// out of the maps' passes, and the FP32 path's FP64-accurate sums run in pairs of
-// floats.  One value per thread and pass with sincospi twiddles and radices up to
+// out of the maps' passes, and the FP32 path's FP64-accurate sums run in FP32
+// (WfSum).  One value per thread and pass with sincospi twiddles and radices up to
 // 7 had taken, 64 maps of 768^2 FP32: 0.40 + 1.64 + 0.61 + 0.08 ms; 8 E/B maps of
 // 375 x 315 FP64: 0.64 + 2.35 + 0.66 + 0.04 ms.
 #include <cuda_runtime.h>
@@ -258,23 +258,22 @@ __device__ __forceinline__ void wf_any_fft(const WfAnyPlan& P, int lgS, V2<T>* A
   }
 }
 
-// Sum of many non-negative products a b with the accuracy of an FP64 sum: FP64, or
-// for FP32 values the exact product (its rounding error from a fused multiply-add)
-// added to a pair of floats by a fast two-sum (exact once the sum is the larger).
-template <typename T> struct WfAnySum;
-template <> struct WfAnySum<double> {
-  double s = 0.0;
-  __device__ __forceinline__ void add(double a, double b) { s = fma(a, b, s); }
-  __device__ __forceinline__ double get() const { return s; }
-};
-template <> struct WfAnySum<float> {
-  float hi = 0.f, lo = 0.f;
-  __device__ __forceinline__ void add(float a, float b) {
-    const float p = __fmul_rn(a, b), e = __fmaf_rn(a, b, -p), t = __fadd_rn(hi, p);
-    lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(p, __fsub_rn(t, hi)), e));
-    hi = t;
+// Sum of many products a b (WfSum), K at a time; those that FP32 does not hold are taken
+// in FP64, in one branch for the K.
+template <typename T> struct WfAnySum {
+  WfSum<T> near;
+  double far = 0.0;
+  template <int K> __device__ __forceinline__ void add(const T (&a)[K], const T (&b)[K]) {
+    bool ok = true;
+#pragma unroll
+    for (int k = 0; k < K; ++k) ok &= near.mul(a[k], b[k]);
+    if (!ok) {
+#pragma unroll
+      for (int k = 0; k < K; ++k)
+        if (!WfSum<T>::holds(a[k] * b[k]) && b[k] != (T)0) far = fma((double)a[k], (double)b[k], far);
+    }
   }
-  __device__ __forceinline__ double get() const { return (double)hi + (double)lo; }
+  __device__ __forceinline__ double get() const { return near.get() + far; }
 };
 
 // Tables of a call.
@@ -434,8 +433,7 @@ k_any_row(const __grid_constant__ WfAnyGeo G, const T* d, const uint8_t* mask, c
           if (q0 + u >= R) break;
           const V2<T> x = v[q0 + u];
           const T r0 = fa[u] - x.x * sc, r1 = fb[u] - x.y * sc, w0 = xa[u] * r0, w1 = xb[u] * r1;
-          acc.add(r0, w0);
-          acc.add(r1, w1);
+          acc.add({r0, r1}, {w0, w1});
           O[at(0, o + (q0 + u) * Ns)] = mk<T>(w0, w1);
         }
       }
@@ -468,7 +466,7 @@ k_any_row(const __grid_constant__ WfAnyGeo G, const T* d, const uint8_t* mask, c
 // column of an even nx, 2 elsewhere).  ppart[b gx + tile] = the tile's sum.  One
 // channel takes the last pass's values as they come; two meet in shared memory.
 template <typename T, int C>
-__global__ void __launch_bounds__(WF_ANY_THREADS)
+__global__ void __launch_bounds__(WF_ANY_THREADS, sizeof(T) == 4 ? 2 : 1)
 k_any_colfwd(const __grid_constant__ WfAnyGeo G, const V2<T>* s, WfAnyTab<T> tab, const V2<T>* scr, V2<T>* grad,
              double* ppart) {
   extern __shared__ __align__(16) unsigned char wf_smem[];
@@ -497,20 +495,25 @@ k_any_colfwd(const __grid_constant__ WfAnyGeo G, const V2<T>* s, WfAnyTab<T> tab
       constexpr int R = decltype(rt)::value;
       const int kx = kx0 + t;
       if (kx >= h1) return;
-      V2<T> sv[R];
-      T a[R];
+      constexpr int U = sizeof(T) == 4 && R > 4 ? 4 : R;  // FP32: four values' loads at once, 64 registers
 #pragma unroll
-      for (int q = 0; q < R; ++q) {
-        const int m = (int)WF_CHK((o + q * Ns) * h1 + kx, nm);
-        sv[q] = __ldg(sb + m);
-        a[q] = __ldg(tab.amp + m);
-      }
+      for (int q0 = 0; q0 < R; q0 += U) {
+        V2<T> sv[U];
+        T a[U];
 #pragma unroll
-      for (int q = 0; q < R; ++q) {
-        const V2<T> g = cscale<T>(v[q], sc);
-        gb[(o + q * Ns) * h1 + kx] = mk<T>((T)2 * (sv[q].x - a[q] * g.x), (T)2 * (sv[q].y - a[q] * g.y));
-        acc.add(sv[q].x, sv[q].x);
-        acc.add(sv[q].y, sv[q].y);
+        for (int u = 0; u < U; ++u) {
+          if (q0 + u >= R) break;
+          const int m = (int)WF_CHK((o + (q0 + u) * Ns) * h1 + kx, nm);
+          sv[u] = __ldg(sb + m);
+          a[u] = __ldg(tab.amp + m);
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          if (q0 + u >= R) break;
+          const V2<T> g = cscale<T>(v[q0 + u], sc);
+          gb[(o + (q0 + u) * Ns) * h1 + kx] = mk<T>((T)2 * (sv[u].x - a[u] * g.x), (T)2 * (sv[u].y - a[u] * g.y));
+          acc.add({sv[u].x, sv[u].y}, {sv[u].x, sv[u].y});
+        }
       }
     };
     wf_any_fft<T, -1, true>(G.py, lgS, A, Bf, tw, at, ld0, stl);
@@ -533,10 +536,7 @@ k_any_colfwd(const __grid_constant__ WfAnyGeo G, const V2<T>* s, WfAnyTab<T> tab
       const V2<T> d1 = mk<T>(r.x * g1.x - r.y * g0.x, r.x * g1.y - r.y * g0.y);   // second row (-s, c)
       gb[m] = mk<T>((T)2 * (s0.x - a0 * d0.x), (T)2 * (s0.y - a0 * d0.y));
       gb[nm + m] = mk<T>((T)2 * (s1.x - a1 * d1.x), (T)2 * (s1.y - a1 * d1.y));
-      acc.add(s0.x, s0.x);
-      acc.add(s0.y, s0.y);
-      acc.add(s1.x, s1.x);
-      acc.add(s1.y, s1.y);
+      acc.add({s0.x, s0.y, s1.x, s1.y}, {s0.x, s0.y, s1.x, s1.y});
     }
   }
   const double tot = wf_rg_block_sum(wm * acc.get(), blockDim.x >> 5);

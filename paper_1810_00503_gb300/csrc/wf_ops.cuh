@@ -587,46 +587,60 @@ __global__ void k_unpack(WfGeo g, int B, const V2<T>* in, V2<T>* out) {
   }
 }
 
+// Running sum of many terms that loses nothing against FP64 additions.  FP64 terms are
+// added as they are.  FP32 ones go to three floats: every term is added to hi by
+// Knuth's two-sum, whose exact error goes to mid the same way and that one's to lo,
+// so that only additions to lo (2^-48 of the sum) round.  A product's own rounding
+// error, exact by a fused multiply-add, starts at mid.  An FP64 instruction holds its
+// unit as long as 64 FP32 ones; a product here takes 22.  wf_eval_any, 64 maps of 768^2:
+// 770 us, against 919 in FP64 and 735 with a pair of floats, whose low part loses the
+// last five bits.
+//
+// mul adds a b and says whether it could: outside [2^-98, 2^100] (or at infinities and
+// NaN) FP32 holds the product or its error no longer, and the caller takes the term in
+// FP64, where holds(a b) is false and b is not 0.
+template <typename T> struct WfSum;
+template <> struct WfSum<float> {
+  float hi = 0.f, mid = 0.f, lo = 0.f;
+  static __device__ __forceinline__ float two_sum(float& s, float p) {  // s += p; the rounding error
+    const float t = __fadd_rn(s, p), z = __fsub_rn(t, s);
+    const float e = __fadd_rn(__fsub_rn(s, __fsub_rn(t, z)), __fsub_rn(p, z));
+    s = t;
+    return e;
+  }
+  __device__ __forceinline__ void add(float p) { lo = __fadd_rn(lo, two_sum(mid, two_sum(hi, p))); }
+  static __device__ __forceinline__ bool holds(float p) { return fabsf(p) >= 0x1p-98f && fabsf(p) <= 0x1p100f; }
+  __device__ __forceinline__ bool mul(float a, float b) {
+    float p = __fmul_rn(a, b), e = __fmaf_rn(a, b, -p);
+    const bool ok = holds(p) || b == 0.f;
+    p = ok ? p : 0.f;
+    e = ok ? e : 0.f;
+    add(p);
+    lo = __fadd_rn(lo, two_sum(mid, e));
+    return ok;
+  }
+  __device__ __forceinline__ double get() const { return (double)hi + ((double)mid + (double)lo); }
+};
+template <> struct WfSum<double> {
+  double s = 0.0;
+  __device__ __forceinline__ void add(double p) { s += p; }
+  static __device__ __forceinline__ bool holds(double) { return true; }
+  __device__ __forceinline__ bool mul(double a, double b) {
+    s = fma(a, b, s);
+    return true;
+  }
+  __device__ __forceinline__ double get() const { return s; }
+};
+
 // Band sums with a bin per thread: what a call with at most WF_BAND_PRIV bands
 // runs.  Every thread walks rows of one column, where the band of a mode changes
-// rarely, and adds a run of equal bands to its own bin when the run ends; the
+// rarely, and adds a run of equal bands (WfSum) to its own bin when the run ends; the
 // threads' bins are added in a fixed order at the end, so the result does not
-// depend on scheduling.  FP32 terms are summed as pairs of floats (Knuth's two-sum,
-// products exact by a fused multiply-add): the accuracy of an FP64 sum without its
-// two lanes an SM.  The per-warp form below takes FP64 adds and shuffles for every
+// depend on scheduling.  The per-warp form below takes FP64 adds and shuffles for every
 // mode: 64 maps of 512^2, ten bands, FP32, derivative: 0.353 ms against 0.043 here
 // (0.020 for its reads at 6.78 TB/s).
 #define WF_BAND_THREADS 128
 #define WF_BAND_PRIV 96  // 96 KB of bins: two blocks an SM
-template <typename T> struct WfBandSum;
-template <> struct WfBandSum<float> {
-  float hi = 0.f, lo = 0.f;
-  __device__ __forceinline__ void add(float p) {
-    const float t = __fadd_rn(hi, p), z = __fsub_rn(t, hi);
-    lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(t, z)), __fsub_rn(p, z)));
-    hi = t;
-  }
-  __device__ __forceinline__ void square(float a) {
-    const float p = __fmul_rn(a, a);
-    lo = __fadd_rn(lo, __fmaf_rn(a, a, -p));
-    add(p);
-  }
-  __device__ __forceinline__ double take() {
-    const double v = (double)hi + (double)lo;
-    hi = lo = 0.f;
-    return v;
-  }
-};
-template <> struct WfBandSum<double> {
-  double s = 0.0;
-  __device__ __forceinline__ void add(double p) { s += p; }
-  __device__ __forceinline__ void square(double a) { s = fma(a, a, s); }
-  __device__ __forceinline__ double take() {
-    const double v = s;
-    s = 0.0;
-    return v;
-  }
-};
 
 // Sums over the half-plane modes of each band, with the full-plane multiplicity
 // (1 on kx = 0 and nx/2, else 2), for rows of hp = nx/2 + 1 modes:
@@ -651,13 +665,17 @@ k_band_priv(int rows, int hp, int tx, const void* s_, const V2<T>* gr, const int
   const V2<T>* gb = MODE == 1 ? gr + (size_t)blockIdx.y * nsp : nullptr;
   constexpr int U = 4;  // rows loaded together
   for (int kx = x0; kx < hp; kx += tx) {
-    const double mult = (kx == 0 || kx == hp - 1) ? 1.0 : 2.0;
+    // the terms' multiplicity and sign: exact factors
+    const T mult = (MODE == 1 ? -1 : 1) * ((kx == 0 || kx == hp - 1) ? 1 : 2);
     int cur = -1;
-    WfBandSum<T> acc;
+    WfSum<T> acc;
     auto apart = [&](double v) {
-      if (cur >= 0) bins[cur * WF_BAND_THREADS] += MODE == 1 ? -mult * v : mult * v;
+      if (cur >= 0) bins[cur * WF_BAND_THREADS] += v;
     };
-    auto flush = [&]() { apart(acc.take()); };
+    auto flush = [&]() {
+      if (cur >= 0) bins[cur * WF_BAND_THREADS] += acc.get();
+      acc = WfSum<T>();
+    };
     for (int j = r0 + y0; j < r1; j += U * ty) {
       int l[U];
       V2<T> x[U], g[U];
@@ -678,22 +696,21 @@ k_band_priv(int rows, int hp, int tx, const void* s_, const V2<T>* gr, const int
           flush();
           cur = lu;
         }
-        // a term that a float sum could not take (the largest, infinities, NaN) goes
-        // to the bin by itself
+        // a term that a float sum could not take (the largest and smallest, infinities,
+        // NaN) goes to the bin by itself
         if constexpr (MODE == 0) {
-          if (sizeof(T) == 8 || (fabs(x[u].x) <= (T)1e15 && fabs(x[u].y) <= (T)1e15)) {
-            acc.square(x[u].x);
-            acc.square(x[u].y);
-          } else {
-            apart(fma((double)x[u].x, (double)x[u].x, (double)x[u].y * (double)x[u].y));
+          const bool okx = acc.mul(x[u].x, mult * x[u].x), oky = acc.mul(x[u].y, mult * x[u].y);
+          if (!(okx && oky)) {
+            if (!okx) apart((double)mult * ((double)x[u].x * x[u].x));
+            if (!oky) apart((double)mult * ((double)x[u].y * x[u].y));
           }
         } else if constexpr (MODE == 1) {
           const T ax = x[u].x - (T)0.5 * g[u].x, ay = x[u].y - (T)0.5 * g[u].y, v = ax * x[u].x + ay * x[u].y;
-          if (sizeof(T) == 8 || fabs(v) <= (T)1e30) acc.add(v);
-          else apart((double)v);
+          if (sizeof(T) == 8 || fabs(v) <= (T)1e30) acc.add(mult * v);
+          else apart((double)mult * v);
         } else {
-          if (MODE == 3 || sizeof(T) == 8 || fabs(x[u].x) <= (T)1e30) acc.add(MODE == 2 ? x[u].x : (T)1);
-          else apart((double)x[u].x);
+          if (MODE == 3 || sizeof(T) == 8 || fabs(x[u].x) <= (T)1e30) acc.add(MODE == 2 ? mult * x[u].x : mult);
+          else apart((double)mult * x[u].x);
         }
       }
     }

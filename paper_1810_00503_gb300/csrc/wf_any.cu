@@ -16,7 +16,7 @@
 //   k_any_prep    once per call: sqrt(P), the rotation's cosine and sine per mode
 //                 and the roots of unity of both lengths, shared by all maps;
 //   k_any_colinv  per column tile: R sqrt(P) s, inverse DFT along y -> scratch;
-//   k_any_row     per pair of rows, a warp each: c2r along x, r = d - x, W r, sum r W r,
+//   k_any_row     per pair of rows, a warp or a block each: c2r along x, r = d - x, W r, sum r W r,
 //                 r2c along x -> scratch;
 //   k_any_colfwd  per column tile: forward DFT along y, sqrt(P) R^T / sqrt N,
 //                 grad, sum of |s|^2 with the half-plane weights;
@@ -49,6 +49,7 @@
 #define WF_ANY_MAXN 1024
 #define WF_ANY_THREADS 512  // most threads of a column block
 #define WF_ANY_ROWW 8       // most warps of a row block
+#define WF_ANY_TEAMT 128    // most threads of a row block of one pair
 
 // One transform length: its passes, with the spans and their reciprocals
 // ceil(2^32 / d) (n / d = umulhi(n, m), exact for n d < 2^32).
@@ -60,7 +61,8 @@ struct WfAnyPlan {
 struct WfAnyGeo {
   int B, C, ny, nx, h1;  // h1 = nx / 2 + 1 half-plane columns
   int tc, lgtc, gx;      // columns of a tile (a power of two), tiles: ceil(h1 / tc)
-  int roww, nrb;         // warps (row pairs) of a row block, row blocks
+  int roww, nrb;         // row pairs of a row block, row blocks
+  int roww_t;            // threads of a row block: a warp a pair, or all for one
   int rpitch;            // shared-memory places of a row sequence
   double inv_sqrt_n;     // (ny nx)^-1/2
   WfAnyPlan py, px;
@@ -369,17 +371,21 @@ k_any_colinv(const __grid_constant__ WfAnyGeo G, const V2<T>* s, WfAnyTab<T> tab
 // conj Z[nx-k]) / 2, B[k] = -i (Z[k] - conj Z[nx-k]) / 2.  An odd last row pairs
 // with itself, its partner's weights 0.  Element e sits at e + e / 16 of the warp's
 // places: the first pass writes with stride R.
-template <typename T>
-__global__ void __launch_bounds__(WF_ANY_ROWW * 32, sizeof(T) == 4 ? 2 : 1)
+// TEAM: a block takes one pair, its threads in place of the warp's lanes.  With few
+// pairs a warp each leaves most of the chip idle and the stage lasts as long as one
+// warp's chain of passes.
+template <typename T, bool TEAM>
+__global__ void __launch_bounds__(TEAM ? WF_ANY_TEAMT : WF_ANY_ROWW * 32, sizeof(T) == 4 && !TEAM ? 2 : 1)
 k_any_row(const __grid_constant__ WfAnyGeo G, const T* d, const uint8_t* mask, const T* Ninv, const V2<T>* twx, V2<T>* scr,
           double* dpart) {
   extern __shared__ __align__(16) unsigned char wf_smem[];
   const int b = blockIdx.y, ny = G.ny, nx = G.nx, h1 = G.h1, rows = G.C * ny, rp = G.rpitch;
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int nteam = TEAM ? 1 : blockDim.x >> 5, team = TEAM ? blockDim.x : 32;  // teams, and threads of one
+  const int lane = TEAM ? threadIdx.x : threadIdx.x & 31, wid = TEAM ? 0 : threadIdx.x >> 5;
   V2<T>* tw = (V2<T>*)wf_smem;
   V2<T>* A = tw + nx + 2 * wid * rp;
   V2<T>* Bf = A + rp;
-  const int pair = blockIdx.x * (blockDim.x >> 5) + wid, ra = 2 * pair;
+  const int pair = blockIdx.x * nteam + wid, ra = 2 * pair;
   const bool on = ra < rows, two = ra + 1 < rows;  // a warp beyond the last pair only meets the block's barriers
   WfAnySum<T> acc;
   if (on) {
@@ -387,13 +393,17 @@ k_any_row(const __grid_constant__ WfAnyGeo G, const T* d, const uint8_t* mask, c
     const size_t pix = ((size_t)b * rows + ra) * nx;
     const char* pw = (const char*)(Ninv + pix);
     const char* pd = (const char*)(d + pix);
-    for (int i = lane * 128; i < (two ? 2 : 1) * nx * (int)sizeof(T); i += 32 * 128) {
+    for (int i = lane * 128; i < (two ? 2 : 1) * nx * (int)sizeof(T); i += team * 128) {
       asm volatile("prefetch.global.L2 [%0];" ::"l"(pw + i));
       if (d) asm volatile("prefetch.global.L2 [%0];" ::"l"(pd + i));
     }
   }
   for (int i = threadIdx.x; i < nx; i += blockDim.x) tw[i] = twx[i];
   __syncthreads();
+  auto sync = [] {
+    if constexpr (TEAM) __syncthreads();  // a block's only pair is never beyond the last
+    else __syncwarp();
+  };
   if (on) {
     const size_t vsz = (size_t)rows * h1, psz = (size_t)rows * nx;
     V2<T>* rowa = scr + (size_t)b * vsz + (size_t)ra * h1;
@@ -438,8 +448,8 @@ k_any_row(const __grid_constant__ WfAnyGeo G, const T* d, const uint8_t* mask, c
         }
       }
     };
-    wf_any_fft<T, +1, false>(G.px, 0, A, Bf, tw, at, ld0, stpix);
-    __syncwarp();
+    wf_any_fft<T, +1, TEAM>(G.px, 0, A, Bf, tw, at, ld0, stpix);
+    sync();
     // forward: the first pass reads O, so the buffers swap roles where O is A
     V2<T>* A2 = O == A ? Bf : A;
     auto ldO = [&](int, int e) { return O[at(0, e)]; };
@@ -448,9 +458,9 @@ k_any_row(const __grid_constant__ WfAnyGeo G, const T* d, const uint8_t* mask, c
 #pragma unroll
       for (int q = 0; q < decltype(rt)::value; ++q) Z[at(0, o + q * Ns)] = v[q];
     };
-    wf_any_fft<T, -1, false>(G.px, 0, A2, O, tw, at, ldO, stZ);
-    __syncwarp();
-    for (int k = lane; k < h1; k += 32) {
+    wf_any_fft<T, -1, TEAM>(G.px, 0, A2, O, tw, at, ldO, stZ);
+    sync();
+    for (int k = lane; k < h1; k += team) {
       const V2<T> zk = Z[at(0, k)], zm = Z[at(0, k == 0 ? 0 : nx - k)];
       rowa[k] = mk<T>((T)0.5 * (zk.x + zm.x), (T)0.5 * (zk.y - zm.y));
       if (two) rowb[k] = mk<T>((T)0.5 * (zk.y + zm.y), (T)0.5 * (zm.x - zk.x));
@@ -600,6 +610,17 @@ template <typename T> static size_t any_col_smem(const WfAnyGeo& G, int tc) {
 template <typename T> static size_t any_row_smem(const WfAnyGeo& G) {
   return ((size_t)G.nx + 2 * (size_t)G.roww * G.rpitch) * sizeof(V2<T>);
 }
+// Butterflies of a transform's widest pass, and the threads for n of them.
+static int any_butterflies(const WfAnyPlan& P) {
+  int n = 0;
+  for (int p = 0; p < P.np; ++p) n = P.LR[p] > n ? P.LR[p] : n;
+  return n;
+}
+static int any_threads(int n, int most) { return n >= most ? most : (n + 31) / 32 * 32; }
+// Row blocks of one pair each up to this many pairs an SM (us a call, a warp a pair -> a
+// block a pair: FP32 12 x 1024 115 -> 106, 600 x 1000 145 -> 128; FP64 60 x 875 210 -> 136,
+// 600 x 1000 300 -> 232); at 480 pairs, 375 values, FP64, it was slower: 191 -> 206.
+#define WF_ANY_TEAM 2
 #define WF_ANY_SMEM2 (113u << 10)
 #define WF_ANY_SMEM1 (226u << 10)
 template <typename T> static void any_tiles(WfAnyGeo& G) {
@@ -622,6 +643,9 @@ template <typename T> static void any_tiles(WfAnyGeo& G) {
   while (G.roww > 1 && any_row_smem<T>(G) > WF_ANY_SMEM2) --G.roww;
   while (G.roww > 1 && (long long)G.B * ((pairs + G.roww - 1) / G.roww) < 2 * WF_SMS) G.roww = (G.roww + 1) / 2;
   G.nrb = (pairs + G.roww - 1) / G.roww;
+  G.roww_t = 32 * G.roww;
+  if (G.roww == 1 && (long long)G.B * pairs <= WF_ANY_TEAM * WF_SMS && any_butterflies(G.px) > 32)
+    G.roww_t = any_threads(any_butterflies(G.px), WF_ANY_TEAMT);
 }
 
 static size_t any_up(size_t x) { return (x + 255) & ~(size_t)255; }
@@ -648,15 +672,18 @@ static cudaError_t wf_any_launch(const WfAnyGeo& G, const void* d, const uint8_t
   auto kf = G.C == 1 ? k_any_colfwd<T, 1> : k_any_colfwd<T, 2>;
   cudaError_t e = cudaFuncSetAttribute(ki, cudaFuncAttributeMaxDynamicSharedMemorySize, WF_ANY_SMEM1);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(kf, cudaFuncAttributeMaxDynamicSharedMemorySize, WF_ANY_SMEM1);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_any_row<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, WF_ANY_SMEM1);
+  auto kr = G.roww_t > 32 * G.roww ? k_any_row<T, true> : k_any_row<T, false>;
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(kr, cudaFuncAttributeMaxDynamicSharedMemorySize, WF_ANY_SMEM1);
   if (e != cudaSuccess) return e;
-  // FP32 threads take 64 registers, so two blocks of 512 fit; FP64 ones up to 128
-  const int tcol = sizeof(T) == 4 || smc > WF_ANY_SMEM2 ? 512 : 256;
+  // FP32 threads take 64 registers, so two blocks of 512 fit; FP64 ones up to 128.  No
+  // more than the widest pass has butterflies: every further warp adds the FP64 steps of
+  // its sums (one map of 12 x 1024, tiles of one column: 134 -> 115 us a call).
+  const int tcol = any_threads(any_butterflies(G.py) * G.C * G.tc, sizeof(T) == 4 || smc > WF_ANY_SMEM2 ? 512 : 256);
   size_t pb = (G.C * nm + 255) / 256;
   if (pb > 8 * WF_SMS) pb = 8 * WF_SMS;
   k_any_prep<T><<<(unsigned)pb, 256, 0, st>>>(G, (const T*)P, tab);
   ki<<<dim3(G.gx, G.B), tcol, smc, st>>>(G, (const V2<T>*)s, tab, (V2<T>*)scr);
-  k_any_row<T><<<dim3(G.nrb, G.B), 32 * G.roww, smr, st>>>(G, (const T*)d, mask, (const T*)Ninv, tab.twx, (V2<T>*)scr, dpart);
+  kr<<<dim3(G.nrb, G.B), G.roww_t, smr, st>>>(G, (const T*)d, mask, (const T*)Ninv, tab.twx, (V2<T>*)scr, dpart);
   kf<<<dim3(G.gx, G.B), tcol, smc, st>>>(G, (const V2<T>*)s, tab, (const V2<T>*)scr, (V2<T>*)grad, ppart);
   k_any_final<<<G.B, 32, 0, st>>>(G.gx, G.nrb, ppart, dpart, chi2);
   return cudaGetLastError();

@@ -63,8 +63,11 @@ static void trim_pools(int dev) {
 // One attempt at an allocation on the current device.
 static cudaError_t allocate(wf_handle* h, void** ptr, size_t bytes, bool pool) {
   if (!pool) return cudaMalloc(ptr, bytes);
-  const cudaError_t e = cudaMallocFromPoolAsync(ptr, bytes, h->pool, h->pool_stream);
-  return e == cudaSuccess ? cudaStreamSynchronize(h->pool_stream) : e;  // usable on every stream from here
+  cudaError_t e = cudaMallocFromPoolAsync(ptr, bytes, h->pool, h->pool_stream);
+  if (e != cudaSuccess) return e;
+  e = cudaStreamSynchronize(h->pool_stream);  // usable on every stream from here
+  if (e != cudaSuccess) cudaFreeAsync(*ptr, h->pool_stream);  // refused, as during a capture: nothing has used it
+  return e;
 }
 
 wf_status wf_alloc(wf_handle* h, void** ptr, size_t bytes, const char* what) {

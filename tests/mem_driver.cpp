@@ -37,7 +37,9 @@ cudaError_t CUDARTAPI cudaDeviceSynchronize() {
 }
 cudaError_t CUDARTAPI cudaStreamCreateWithFlags(cudaStream_t* s, unsigned) { *s = (cudaStream_t)malloc(1); return cudaSuccess; }
 cudaError_t CUDARTAPI cudaStreamDestroy(cudaStream_t s) { free(s); return cudaSuccess; }
-cudaError_t CUDARTAPI cudaStreamSynchronize(cudaStream_t) { return cudaSuccess; }
+cudaError_t CUDARTAPI cudaStreamSynchronize(cudaStream_t) {
+  return g_sync_fails ? cudaErrorStreamCaptureUnsupported : cudaSuccess;
+}
 cudaError_t CUDARTAPI cudaMemPoolCreate(cudaMemPool_t* p, const cudaMemPoolProps* pr) {
   *p = (cudaMemPool_t) new Pool{pr->location.id, 0, 0};
   return cudaSuccess;
@@ -205,12 +207,28 @@ static int trims() {
   return 0;
 }
 
+// An allocation whose wait is refused (a capture in progress) leaves nothing behind.
+static int refused() {
+  wf_handle h;
+  open(&h, 0);
+  void* a;
+  g_sync_fails = true;
+  CHECK(wf_alloc(&h, &a, 1 << 20, "a") == WF_ECUDA && !a && h.used == 0 && g_live.empty());
+  g_sync_fails = false;
+  CHECK(wf_alloc(&h, &a, 1 << 20, "a") == WF_OK);
+  wf_free(&h, a);
+  CHECK(h.used == 0 && g_live.empty());
+  wf_mem_close(&h);
+  return 0;
+}
+
 int main(int argc, char** argv) {
   const std::string t = argc > 1 ? argv[1] : "";
   if (t == "other_device") return other_device();
   if (t == "failed_wait") return failed_wait();
   if (t == "current_device") return current_device();
   if (t == "trims") return trims();
+  if (t == "refused") return refused();
   printf("unknown test\n");
   return 2;
 }

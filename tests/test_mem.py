@@ -23,7 +23,7 @@ def driver(tmp_path_factory):
     return exe
 
 
-@pytest.mark.parametrize("what", ["other_device", "failed_wait", "current_device", "trims"])
+@pytest.mark.parametrize("what", ["other_device", "failed_wait", "current_device", "trims", "refused"])
 def test_memory_of_a_handle(driver, what):
     r = subprocess.run([driver, what], capture_output=True, text=True, timeout=60)
     assert r.returncode == 0, r.stdout

@@ -402,7 +402,8 @@ def run_hetero(args, dev, count=256, n_bands=10, sizes=(64, 128, 256, 512, 1024)
     """Heterogeneous batch: `count` independent maps of n in {64, 128, 256,
     512, 1024} (uneven masks, noise levels and spectral slopes), one problem
     per size, all solved as one batch by wf_map_solve_many (each iteration one
-    set of seven launches shared by every size, one CUDA graph per round) to
+    set of seven launches shared by the sizes, plus three for each size that fills
+    the chip alone, one CUDA graph per round) to
     ||g|| / ||g0|| < 1e-6 in mixed precision;
     then d chi^2 / d log q for n_bands log-spaced bands at the solutions
     through the adjoint stage (wf_eval_bands)."""
@@ -455,8 +456,9 @@ def run_hetero(args, dev, count=256, n_bands=10, sizes=(64, 128, 256, 512, 1024)
             "evals_per_s": evals / dt, "stop": "||g||/||g0|| < 1e-6", "statuses": statuses,
             "dchi2_dlogq": {"bands": n_bands, "ms_per_batch": dq_dt * 1e3, "maps_per_s": count / dq_dt},
             "note": "one problem per size, all sizes solved as one batch by wf_map_solve_many: each iteration "
-                    "is seven launches shared by the five sizes (register-resident stages, tile widths tuned per size), each "
-                    "round of 32 iterations one graph launch; a 2-iteration solve first tunes and sets up the solvers"}
+                    "is seven launches shared by the sizes, plus three for each that fills the chip alone "
+                    "(register-resident stages, tile widths tuned per size), each round of 32 iterations one "
+                    "graph launch; a 2-iteration solve first tunes and sets up the solvers"}
 
 
 def run_alu_peaks():
@@ -597,10 +599,10 @@ def iteration_flops(n, m):
     complex FFT of length L: two real 2-D transforms; 5m + 9 complex dot
     products or real-coefficient axpys per packed value, 4 flops each; about
     10 flops per value for the per-mode and per-pixel steps), which
-    overcounts the radix-8/16 butterflies.  Returns (flops, source)."""
+    overcounts the butterflies.  Returns (flops, source)."""
     import math
     if (n, m) in FP64_ITERATION_FLOPS_COUNTED:
-        return FP64_ITERATION_FLOPS_COUNTED[(n, m)], "ncu FP64 instruction counters of the three-pass stages"
+        return FP64_ITERATION_FLOPS_COUNTED[(n, m)], "ncu FP64 instruction counters, variant 3122"
     h = n // 2
     fft = 5 * (h * n * math.log2(n) + n * h * math.log2(h))
     vals = n * h

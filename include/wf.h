@@ -364,9 +364,10 @@ wf_status wf_solver_history(const wf_problem* p, double* out, int* counts);
  * the blocks of every problem's own grid, each block running the
  * single-problem kernel at its place in its problem's grid, every problem on
  * the register-resident column and row stages with its own tile widths (tuned
- * per shape when opts->autotune, else the widest: variant 2111), so each map
- * ends exactly where its problem solved alone with the
- * variant its stats report ends.  Otherwise every problem is tuned and
+ * per shape when opts->autotune, else the widest: variant 2111).  A problem of
+ * 1024 column tiles or more, which fills the chip alone, runs its three FFT
+ * stages in launches of its own beside the shared ones.  Each map ends exactly
+ * where its problem solved alone with the variant its stats report ends.  Otherwise every problem is tuned and
  * runs its own kernels, a parallel branch per problem.  opts->check_every
  * iterations are captured in one CUDA graph, so that each round of the batch
  * is one graph launch (plain launches when opts->use_graphs is 0) and one

@@ -26,7 +26,7 @@
 //
 // Measured, 120 maps of 1024^2, FP32 (bytes at 6.78 TB/s: 0.15, 0.30 and 0.22
 // ms): inverse column stage 0.466 -> 0.248 ms, row stage with data 0.533 -> 0.330
-// ms, forward column stage 0.626 -> 0.393 ms; the objective pass 1.637 -> 0.985
+// ms, forward column stage 0.626 -> 0.393 ms; the objective pass 1.637 -> 1.00
 // ms.  53 E/B maps of 512^2, Hessian-vector product: 0.448 -> 0.272 ms.
 #pragma once
 #include "wf_ops.cuh"

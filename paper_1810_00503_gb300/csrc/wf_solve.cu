@@ -1382,7 +1382,7 @@ static cudaError_t any_refresh(wf_problem* p, cudaStream_t st) {
 
 // One L-BFGS iteration of several problems in shared launches (see
 // WfMultiArgs): the five kernels of iteration() plus the active counters'
-// reset and the scalar step, seven launches whatever the number of problems.  A
+// reset and the scalar step, seven launches whatever the number of small problems.  A
 // problem whose column stage alone has WF_MULTI_SOLO blocks runs its FFT stages in
 // launches of its own: they fill the chip, and are not held to the registers and
 // shared memory of the other lengths (64^2 to 1024^2, 48 maps each: 14.2 against
@@ -1423,7 +1423,7 @@ static cudaError_t multi_iteration(const WfMultiArgs& a, const WfMultiScalar& ms
 // solved as one batch.  Every problem is started on its own stream (first
 // gradient).  When the problems share the working type and C (and no FFT-stage
 // variant is forced), each iteration of the whole batch is seven shared
-// launches (multi_iteration), every problem on the register-resident stages of
+// launches, and three for every large problem (multi_iteration), every problem on the register-resident stages of
 // WF_MULTI_VARIANT with its own tuned tile widths; otherwise each problem is
 // tuned freely and runs its own kernels, as a parallel branch per problem.  check_every iterations are
 // captured in one CUDA graph, so that each round is one graph launch for the

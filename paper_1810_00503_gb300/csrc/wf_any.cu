@@ -260,20 +260,17 @@ __device__ __forceinline__ void wf_any_fft(const WfAnyPlan& P, int lgS, V2<T>* A
   }
 }
 
-// Sum of many products a b (WfSum), K at a time; those that FP32 does not hold are taken
-// in FP64, in one branch for the K.
+// Sum of many products a b (WfSum), two at a time; a pair that FP32 does not hold is
+// taken in FP64, out of line: inlined it is predicated, and instructions that do nothing
+// hold the FP64 unit all the same (64 maps of 768^2: 908 us a call against 751).
+template <typename T> static __device__ __noinline__ double wf_any_far(double far, T a0, T b0, T a1, T b1) {
+  return fma((double)a1, (double)b1, fma((double)a0, (double)b0, far));
+}
 template <typename T> struct WfAnySum {
   WfSum<T> near;
   double far = 0.0;
-  template <int K> __device__ __forceinline__ void add(const T (&a)[K], const T (&b)[K]) {
-    bool ok = true;
-#pragma unroll
-    for (int k = 0; k < K; ++k) ok &= near.mul(a[k], b[k]);
-    if (!ok) {
-#pragma unroll
-      for (int k = 0; k < K; ++k)
-        if (!WfSum<T>::holds(a[k] * b[k]) && b[k] != (T)0) far = fma((double)a[k], (double)b[k], far);
-    }
+  __device__ __forceinline__ void add(const T (&a)[2], const T (&b)[2]) {
+    if (!wf_sum_products(near, a, b)) far = wf_any_far<T>(far, a[0], b[0], a[1], b[1]);
   }
   __device__ __forceinline__ double get() const { return near.get() + far; }
 };
@@ -476,7 +473,7 @@ k_any_row(const __grid_constant__ WfAnyGeo G, const T* d, const uint8_t* mask, c
 // column of an even nx, 2 elsewhere).  ppart[b gx + tile] = the tile's sum.  One
 // channel takes the last pass's values as they come; two meet in shared memory.
 template <typename T, int C>
-__global__ void __launch_bounds__(WF_ANY_THREADS, sizeof(T) == 4 ? 2 : 1)
+__global__ void __launch_bounds__(WF_ANY_THREADS, sizeof(T) == 4 ? 2 : 0)
 k_any_colfwd(const __grid_constant__ WfAnyGeo G, const V2<T>* s, WfAnyTab<T> tab, const V2<T>* scr, V2<T>* grad,
              double* ppart) {
   extern __shared__ __align__(16) unsigned char wf_smem[];
@@ -546,7 +543,8 @@ k_any_colfwd(const __grid_constant__ WfAnyGeo G, const V2<T>* s, WfAnyTab<T> tab
       const V2<T> d1 = mk<T>(r.x * g1.x - r.y * g0.x, r.x * g1.y - r.y * g0.y);   // second row (-s, c)
       gb[m] = mk<T>((T)2 * (s0.x - a0 * d0.x), (T)2 * (s0.y - a0 * d0.y));
       gb[nm + m] = mk<T>((T)2 * (s1.x - a1 * d1.x), (T)2 * (s1.y - a1 * d1.y));
-      acc.add({s0.x, s0.y, s1.x, s1.y}, {s0.x, s0.y, s1.x, s1.y});
+      acc.add({s0.x, s0.y}, {s0.x, s0.y});
+      acc.add({s1.x, s1.y}, {s1.x, s1.y});
     }
   }
   const double tot = wf_rg_block_sum(wm * acc.get(), blockDim.x >> 5);

@@ -593,12 +593,12 @@ __global__ void k_unpack(WfGeo g, int B, const V2<T>* in, V2<T>* out) {
 // so that only additions to lo (2^-48 of the sum) round.  A product's own rounding
 // error, exact by a fused multiply-add, starts at mid.  An FP64 instruction holds its
 // unit as long as 64 FP32 ones; a product here takes 22.  wf_eval_any, 64 maps of 768^2:
-// 770 us, against 919 in FP64 and 735 with a pair of floats, whose low part loses the
+// 751 us, against 919 in FP64 and 735 with a pair of floats, whose low part loses the
 // last five bits.
 //
-// mul adds a b and says whether it could: outside [2^-98, 2^100] (or at infinities and
-// NaN) FP32 holds the product or its error no longer, and the caller takes the term in
-// FP64, where holds(a b) is false and b is not 0.
+// mul adds a b and says whether that was right: outside [2^-98, 2^100] (or at infinities
+// and NaN) FP32 holds the product or its error no longer.  wf_sum_products then leaves
+// the sum as it was and says so, and the caller takes its products in FP64.
 template <typename T> struct WfSum;
 template <> struct WfSum<float> {
   float hi = 0.f, mid = 0.f, lo = 0.f;
@@ -609,28 +609,32 @@ template <> struct WfSum<float> {
     return e;
   }
   __device__ __forceinline__ void add(float p) { lo = __fadd_rn(lo, two_sum(mid, two_sum(hi, p))); }
-  static __device__ __forceinline__ bool holds(float p) { return fabsf(p) >= 0x1p-98f && fabsf(p) <= 0x1p100f; }
   __device__ __forceinline__ bool mul(float a, float b) {
-    float p = __fmul_rn(a, b), e = __fmaf_rn(a, b, -p);
-    const bool ok = holds(p) || b == 0.f;
-    p = ok ? p : 0.f;
-    e = ok ? e : 0.f;
+    const float p = __fmul_rn(a, b);
     add(p);
-    lo = __fadd_rn(lo, two_sum(mid, e));
-    return ok;
+    lo = __fadd_rn(lo, two_sum(mid, __fmaf_rn(a, b, -p)));
+    return (fabsf(p) >= 0x1p-98f && fabsf(p) <= 0x1p100f) || b == 0.f;
   }
   __device__ __forceinline__ double get() const { return (double)hi + ((double)mid + (double)lo); }
 };
 template <> struct WfSum<double> {
   double s = 0.0;
   __device__ __forceinline__ void add(double p) { s += p; }
-  static __device__ __forceinline__ bool holds(double) { return true; }
   __device__ __forceinline__ bool mul(double a, double b) {
     s = fma(a, b, s);
     return true;
   }
   __device__ __forceinline__ double get() const { return s; }
 };
+template <typename T, int K>
+__device__ __forceinline__ bool wf_sum_products(WfSum<T>& sum, const T (&a)[K], const T (&b)[K]) {
+  WfSum<T> t = sum;
+  bool ok = true;
+#pragma unroll
+  for (int k = 0; k < K; ++k) ok &= t.mul(a[k], b[k]);
+  if (ok) sum = t;
+  return ok;
+}
 
 // Band sums with a bin per thread: what a call with at most WF_BAND_PRIV bands
 // runs.  Every thread walks rows of one column, where the band of a mode changes
@@ -699,11 +703,8 @@ k_band_priv(int rows, int hp, int tx, const void* s_, const V2<T>* gr, const int
         // a term that a float sum could not take (the largest and smallest, infinities,
         // NaN) goes to the bin by itself
         if constexpr (MODE == 0) {
-          const bool okx = acc.mul(x[u].x, mult * x[u].x), oky = acc.mul(x[u].y, mult * x[u].y);
-          if (!(okx && oky)) {
-            if (!okx) apart((double)mult * ((double)x[u].x * x[u].x));
-            if (!oky) apart((double)mult * ((double)x[u].y * x[u].y));
-          }
+          if (!wf_sum_products<T, 2>(acc, {x[u].x, x[u].y}, {mult * x[u].x, mult * x[u].y}))
+            apart((double)mult * fma((double)x[u].x, (double)x[u].x, (double)x[u].y * (double)x[u].y));
         } else if constexpr (MODE == 1) {
           const T ax = x[u].x - (T)0.5 * g[u].x, ay = x[u].y - (T)0.5 * g[u].y, v = ax * x[u].x + ay * x[u].y;
           if (sizeof(T) == 8 || fabs(v) <= (T)1e30) acc.add(mult * v);

@@ -588,9 +588,9 @@ def run_eb_bandpower(args, dev, n=512, n_bands=8, n_sim=20, n_fd=2):
 FP64_PEAK_TFLOPS = 1.25  # GB300 nominal dense FP64
 
 
-# FP64 FLOPs of one L-BFGS iteration counted by ncu on the FP64 path (DFMA as
-# two; profiles/fp64_iteration_cmb1024_counters.md), per (n, m).
-FP64_ITERATION_FLOPS_COUNTED = {(1024, 10): 158.3e6}
+# FP64 FLOPs of one L-BFGS iteration with a full history counted by ncu on the FP64
+# path (DFMA as two; profiles/fp64_iteration_cmb1024_counters.md), per (n, m).
+FP64_ITERATION_FLOPS_COUNTED = {(1024, 10): 216.3e6}
 
 
 def iteration_flops(n, m):
@@ -638,7 +638,7 @@ def run_fp64_reference(args, dev, cert_tol=1e-4, fp64_peak=None):
     stream = torch.cuda.Stream(device=dev)
     with torch.cuda.stream(stream):
         p64.start(gtol_rel=0.0, max_iter=1 << 30, check_every=1)
-        p64.step(5)
+        p64.step(args.m + 2)  # a full history
         e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
         e0.record(stream)
         p64.step(args.steps, sync=False)
